@@ -60,6 +60,7 @@ struct FftRes {
   double2* tw_d = nullptr;
   int* pos = nullptr;
   int* freq = nullptr;
+  float4* tw2 = nullptr;
 };
 
 // a packed y-DFT matrix of the reduced-precision form and what it was built for
@@ -81,6 +82,7 @@ struct Dir {
   int start[3] = {0, 0, 0}, r[3] = {0, 0, 0}, guard[3] = {0, 0, 0};
   int Tq_box_lo_z = 0, Tq_bz = 0, Tq_start_z = 0, Tq_nout = 0, Tq_prefilter = -1, Tq_Q[2] = {0, 0};
   int Tq_kind = 0;             // 0: S (potential); 1: rows of -N (componentwise field variant)
+  int Tq_stride = 0;           // planes per output (t_stride)
   float* Tq = nullptr;
   float2* YC = nullptr;
   float* C = nullptr;
@@ -422,23 +424,72 @@ std::vector<int> plan_radices(int L) {
   return best;
 }
 
+// Shared-memory wavefronts of all stage loads of a plan on pair lines (fft2.cuh):
+// one 16-byte access per butterfly point, served eight lanes at a time.
+long long pair_wavefronts(int L, const std::vector<int>& radix) {
+  long long total = 0;
+  int Lb = L;
+  for (int R : radix) {
+    const int M = Lb / R, per_line = L / R;
+    for (int w = 0; w < per_line; w += 8) {
+      int count[8] = {0}, worst = 0;
+      for (int b = w; b < std::min(w + 8, per_line); ++b) worst = std::max(worst, ++count[(b / M * Lb + b % M) & 7]);
+      total += (long long)worst * R;
+    }
+    Lb /= R;
+  }
+  return total;
+}
+
+// The plan of a pass on pair lines: radices up to 12 (a butterfly holds both
+// lines, 4 R registers; 15 and 16 leave too few warps or spill), the fewest
+// stages, of those orders the fewest modelled wavefronts, then the smallest
+// largest radix.  Measured in the y pass: 160 = 4 8 5 13 us against 16 10 20 us,
+// 540 = 12 9 5 92 us against 4 9 15 94 us and 10 6 9 98 us.
+std::vector<int> plan_pair_radices(int L) {
+  constexpr int max_r = 12;
+  std::vector<int> cur, best;
+  radix_search(L, max_r, cur, best);
+  if (best.empty()) return best;
+  std::vector<std::vector<int>> orders;
+  cur.clear();
+  radix_orders(L, (int)best.size(), cur, orders);
+  long long best_key = -1;
+  for (const auto& o : orders) {
+    const int m = *std::max_element(o.begin(), o.end());
+    if (m > max_r) continue;
+    const long long key = pair_wavefronts(L, o) * 64 + m;
+    if (best_key < 0 || key < best_key) {
+      best_key = key;
+      best = o;
+    }
+  }
+  return best;
+}
+
 // ------------------------------------------------------------ autotuned plans
 // Process-wide radix order per transform length, chosen by mm_autotune from
 // timed runs of the pass kernels; the planner's model choice otherwise.
+// `pairs`: it also ran faster than the planner's choice for pair lines, so the
+// passes on pair lines take it too.
+struct Tuned {
+  std::vector<int> radix;
+  bool pairs;
+};
 std::mutex g_tune_mu;
-std::map<int, std::vector<int>> g_tuned;
+std::map<int, Tuned> g_tuned;
 
-bool tuned_plan(int L, std::vector<int>* out) {
+bool tuned_plan(int L, std::vector<int>* out, bool pairs = false) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
   auto it = g_tuned.find(L);
-  if (it == g_tuned.end()) return false;
-  if (out) *out = it->second;
+  if (it == g_tuned.end() || (pairs && !it->second.pairs)) return false;
+  if (out) *out = it->second.radix;
   return true;
 }
 
-void set_tuned_plan(int L, const std::vector<int>& r) {
+void set_tuned_plan(int L, const std::vector<int>& r, bool pairs) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  g_tuned[L] = r;
+  g_tuned[L] = Tuned{r, pairs};
 }
 
 // The candidates an autotuner times for length L: the model's choice first,
@@ -463,9 +514,10 @@ std::vector<std::vector<int>> plan_candidates(int L, int k) {
 }
 
 // FFT resources of length L (plan, twiddle and position tables), cached per
-// context; the plan is the autotuned one when mm_autotune has chosen it.
-mm_status get_fft(mm_ctx* ctx, int L, FftTables* out) {
-  const int key = L;
+// context (pairs: for the passes on pair lines, under -L); the plan is the
+// autotuned one when mm_autotune has chosen it.
+mm_status get_fft(mm_ctx* ctx, int L, FftTables* out, bool pairs = false) {
+  const int key = pairs ? -L : L;
   auto it = ctx->ffts.find(key);
   if (it != ctx->ffts.end()) {
     *out = it->second.t;
@@ -479,7 +531,7 @@ mm_status get_fft(mm_ctx* ctx, int L, FftTables* out) {
   if (r != 1) return fail(ctx, MM_EINVAL, "FFT length is not 2^a 3^b 5^c");
   (void)p2; (void)p3; (void)p5;
   std::vector<int> radix;
-  if (!tuned_plan(L, &radix)) radix = plan_radices(L);
+  if (!tuned_plan(L, &radix, pairs)) radix = pairs ? plan_pair_radices(L) : plan_radices(L);
   if (radix.empty() || (int)radix.size() > kMaxStages)
     return fail(ctx, MM_ENOTSUP, "FFT length has too many factors");
   FftPlanDev P{};
@@ -516,6 +568,21 @@ mm_status get_fft(mm_ctx* ctx, int L, FftTables* out) {
     twd.push_back(make_double2(1.0, 0.0));
   }
   const size_t ntw = twf.size();
+  // the pair table: rows of (c, c, s, s), pitch odd
+  std::vector<float4> tw2;
+  for (int s = 0; s < P.nstages; ++s) {
+    const int r = P.radix[s], M = P.blocklen[s] / r, pitch = (r - 1) | 1;
+    R.t.tw2_off[s] = (int)tw2.size();
+    if (M == 1) continue;
+    tw2.resize(tw2.size() + (size_t)M * pitch, make_float4(0.f, 0.f, 0.f, 0.f));
+    for (int n1 = 0; n1 < M; ++n1)
+      for (int k = 1; k < r; ++k) {
+        const float2 w = twf[P.stw_off[s] + (k - 1) * M + n1];
+        tw2[R.t.tw2_off[s] + n1 * pitch + k - 1] = make_float4(w.x, w.x, w.y, w.y);
+      }
+  }
+  R.t.ntw2 = (int)tw2.size();
+  if (tw2.empty()) tw2.resize(1, make_float4(0.f, 0.f, 0.f, 0.f));
   std::vector<int> pos(L), freq(L);
   for (int k = 0; k < L; ++k) {
     int p = 0, rem = k, B = L;
@@ -530,15 +597,18 @@ mm_status get_fft(mm_ctx* ctx, int L, FftTables* out) {
   }
   CKS(alloc(ctx, (void**)&R.tw_f, sizeof(float2) * ntw));
   CKS(alloc(ctx, (void**)&R.tw_d, sizeof(double2) * ntw));
+  CKS(alloc(ctx, (void**)&R.tw2, sizeof(float4) * tw2.size()));
   CKS(alloc(ctx, (void**)&R.pos, sizeof(int) * L));
   CKS(alloc(ctx, (void**)&R.freq, sizeof(int) * L));
   CK(cudaMemcpy(R.tw_f, twf.data(), sizeof(float2) * ntw, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(R.tw_d, twd.data(), sizeof(double2) * ntw, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(R.tw2, tw2.data(), sizeof(float4) * tw2.size(), cudaMemcpyHostToDevice));
   CK(cudaMemcpy(R.pos, pos.data(), sizeof(int) * L, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(R.freq, freq.data(), sizeof(int) * L, cudaMemcpyHostToDevice));
   R.t.plan = P;
   R.t.tw_f = R.tw_f;
   R.t.tw_d = R.tw_d;
+  R.t.tw2 = R.tw2;
   R.t.pos = R.pos;
   R.t.freq = R.freq;
   ctx->ffts[key] = R;
@@ -677,7 +747,8 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   Magnet& S = ctx->mag[s];
   const int n_out = D->r[2];
   const int bz = D->box_len[2];
-  if (D->Tq && D->Tq_box_lo_z == D->box_lo[2] && D->Tq_bz == bz && D->Tq_start_z == D->start[2] &&
+  const int tstride = t_stride(S.nz, kind == 0 && !S.thick);  // the fused y pass reads it, or the plane mixing pass
+  if (D->Tq && D->Tq_stride == tstride && D->Tq_box_lo_z == D->box_lo[2] && D->Tq_bz == bz && D->Tq_start_z == D->start[2] &&
       D->Tq_nout == n_out && D->Tq_prefilter == D->prefilter && D->Tq_Q[0] == S.Qx &&
       D->Tq_Q[1] == S.Qy && D->Tq_kind == kind)
     return MM_OK;
@@ -685,7 +756,9 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   CKS(get_fft(ctx, S.Qx, &fx));
   CKS(get_fft(ctx, S.Qy, &fy));
   const size_t qsize = (size_t)S.kxh * S.kyq;
-  CKS(ensure_buf(ctx, &D->Tq, &D->Tq_bytes, sizeof(float) * (size_t)(kind ? 3 : 1) * n_out * S.nz * 3 * qsize));
+  const size_t tbytes = sizeof(float) * quad_floats((kind ? 3 : 1) * n_out * tstride, S.kxh, S.kyq);
+  CKS(ensure_buf(ctx, &D->Tq, &D->Tq_bytes, tbytes));
+  CK(cudaMemsetAsync(D->Tq, 0, tbytes, ctx->st));  // the padding of the quads
   // z mixing matrix: rows = output planes, columns = box planes
   std::vector<double> W((size_t)n_out * bz, 0.0);
   double h[kFirHalf + 1];
@@ -708,7 +781,7 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   const double scale = S.Ms / ((double)S.Qx * S.Qy);
   if (kind == 0)
     CK(build_T_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], scale, D->box_lo[2], bz, n_out, ctx->W_dev, D->Tq,
-                       ctx->gen_work, ctx->gen_q, ctx->st));
+                       tstride, ctx->gen_work, ctx->gen_q, ctx->st));
   else  // H = -N M
     CK(build_TN_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], -scale, D->box_lo[2], bz, n_out, ctx->W_dev, D->Tq,
                         ctx->gen_work, ctx->gen_q, ctx->st));
@@ -721,6 +794,7 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   D->Tq_Q[0] = S.Qx;
   D->Tq_Q[1] = S.Qy;
   D->Tq_kind = kind;
+  D->Tq_stride = tstride;
   return MM_OK;
 }
 
@@ -859,7 +933,9 @@ mm_status ensure_plan(mm_ctx* ctx) {
       CKS(alloc(ctx, (void**)&S.X1, sizeof(float2) * 3 * S.nz * S.kxh * (size_t)S.ny));
       CKS(alloc(ctx, (void**)&S.YH, sizeof(float2) * 3 * S.nz * S.kxh * (size_t)S.ny));
       if (!S.zfft) {
-        CKS(alloc(ctx, (void**)&S.Nq, sizeof(float) * 6 * S.nz * qsize));
+        const size_t nbytes = sizeof(float) * quad_floats(6 * S.nz, S.kxh, S.kyq);
+        CKS(alloc(ctx, (void**)&S.Nq, nbytes));
+        CK(cudaMemsetAsync(S.Nq, 0, nbytes, ctx->st));  // the padding of the quads
       } else {
         CKS(alloc(ctx, (void**)&S.N3, sizeof(float) * 6 * qsize * S.kzq));
         CKS(alloc(ctx, (void**)&S.S3, sizeof(float) * 3 * qsize * S.kzq));
@@ -1019,7 +1095,7 @@ mm_status run_source_passes(mm_ctx* ctx, const float* in[2], const int* which, i
       YJob& J = L.job[nj];
       J.in = S.X1;
       J.nz = S.nz; J.ny = S.ny; J.kxh = S.kxh; J.kyq = S.kyq;
-      CKS(get_fft(ctx, S.Qy, &J.fy));
+      CKS(get_fft(ctx, S.Qy, &J.fy, true));
       J.do_H = (what[i] & 1) ? 1 : 0;
       J.Nq = S.Nq;
       J.outH = S.YH;
@@ -1115,7 +1191,7 @@ mm_status run_source_passes(mm_ctx* ctx, const float* in[2], const int* which, i
         M.outH = S.Z3H;
         M.outC = do_C ? D->Z3C : nullptr;
         Lm.tile_start[nm] = tm;
-        tm += S.kxh * zmix_tiles(S.kyq, M.nH + M.n_out);
+        tm += zmix_tiles(S.kxh, S.kyq);
         ++nm;
       }
       if (mixed) {
@@ -1733,7 +1809,7 @@ void mm_destroy(mm_ctx* ctx) {
     cudaFree(M.Bprev); cudaFree(M.Bdot); cudaFree(M.Heddy);
   }
   for (auto& kv : ctx->ffts) {
-    cudaFree(kv.second.tw_f); cudaFree(kv.second.tw_d); cudaFree(kv.second.pos); cudaFree(kv.second.freq);
+    cudaFree(kv.second.tw_f); cudaFree(kv.second.tw_d); cudaFree(kv.second.tw2); cudaFree(kv.second.pos); cudaFree(kv.second.freq);
   }
   cudaFree(ctx->gen_work); cudaFree(ctx->gen_q); cudaFree(ctx->W_dev); cudaFree(ctx->dc_buf);
   cudaFree(ctx->fd4_C); cudaFree(ctx->fd4_V);
@@ -2249,7 +2325,7 @@ mm_status mm_compute_stray_field_componentwise(mm_ctx* ctx, int src, float* H_de
     M.in = S.cw_Y; M.nz = S.nz; M.kxh = S.kxh; M.Qy = S.Qy; M.kyq = S.kyq;
     M.Nq = S.Nq; M.Tq = D.Tq; M.nH = 0; M.n_out = PC; M.outH = nullptr; M.outC = D.Z3C;
     M.field_nbox = nb;
-    L.tile_start[1] = S.kxh * zmix_tiles(S.kyq, PC);
+    L.tile_start[1] = zmix_tiles(S.kxh, S.kyq);
     Timer t(ctx, 8);
     CK(launch_zmix3(L, st));
   }
@@ -2596,12 +2672,14 @@ mm_status mm_assign_lanes(const double* cost, int npairs, int nlanes, int* lane_
 // Drops this context's tables of length L (after its work has drained), so
 // the next launch builds them from the current plan of L.
 static mm_status drop_fft(mm_ctx* ctx, int L) {
-  auto it = ctx->ffts.find(L);
-  if (it == ctx->ffts.end()) return MM_OK;
   CK(cudaStreamSynchronize(ctx->st));
   if (ctx->side) CK(cudaStreamSynchronize(ctx->side));
-  cudaFree(it->second.tw_f); cudaFree(it->second.tw_d); cudaFree(it->second.pos); cudaFree(it->second.freq);
-  ctx->ffts.erase(it);
+  for (int key : {L, -L}) {
+    auto it = ctx->ffts.find(key);
+    if (it == ctx->ffts.end()) continue;
+    cudaFree(it->second.tw_f); cudaFree(it->second.tw_d); cudaFree(it->second.tw2); cudaFree(it->second.pos); cudaFree(it->second.freq);
+    ctx->ffts.erase(it);
+  }
   return MM_OK;
 }
 
@@ -2653,10 +2731,13 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
     }
     const auto cands = plan_candidates(L, candidates);
     if (cands.empty()) continue;
-    double best_ms = 0.0;
+    double best_ms = 0.0, own_ms = 0.0;
     size_t best = 0;
+    // the planner's choices first: the passes on pair lines have one of their own
+    if ((st = run()) != MM_OK) break;
+    for (int cls : kv.second) own_ms += ctx->t_ms[cls];
     for (size_t c = 0; c < cands.size() && cands.size() > 1; ++c) {
-      set_tuned_plan(L, cands[c]);
+      set_tuned_plan(L, cands[c], true);
       if ((st = drop_fft(ctx, L)) != MM_OK) break;
       if ((st = run()) != MM_OK) break;
       double ms = 0.0;
@@ -2667,7 +2748,7 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
       }
     }
     if (st != MM_OK) break;
-    set_tuned_plan(L, cands[best]);
+    set_tuned_plan(L, cands[best], cands.size() > 1 && best_ms < own_ms);
     if ((st = drop_fft(ctx, L)) != MM_OK) break;
     if (n_tuned) ++*n_tuned;
   }

@@ -25,6 +25,7 @@
 #include <algorithm>
 
 #include "fft.cuh"
+#include "fft2.cuh"
 #include "mm_internal.h"
 #include "prefilter.cuh"
 #include "umma.cuh"
@@ -254,99 +255,45 @@ static cudaError_t prep(const void* f, size_t smem) {
 }
 
 // ------------------------------------------------------------------ direct z sum
-// The thin-film plane mixing of Sec. III.A for sources of up to kMaxNzDirect
-// layers.  CTA -> (kx, a chunk of kZMixChunk frequency pairs ky, Qy - ky): the
-// input planes of the chunk are staged in shared memory once, then each warp
-// takes one output plane at a time with one frequency pair per lane, so the
-// kernel-spectrum loads and the output stores are coalesced runs and the
-// inputs are read from shared memory instead of again from L2 for every
-// output plane.  (Staging inputs and looping over all outputs inside one
-// thread measured 1.3-2.7x slower than streaming; this layout keeps a warp
-// per output plane.)
+// The plane mixing of Sec. III.A for sources of up to kMaxNzDirect layers.
+// CTA -> (two kx columns, a chunk of kZMixChunk frequency pairs ky, Qy - ky):
+// the input planes of the chunk are staged in shared memory once, both columns
+// packed (fft2.cuh), then each warp takes output planes with one frequency pair
+// per lane.  A warp takes two coefficient planes, or the three demag planes of
+// one layer, at a time: every staged input then serves two or three outputs,
+// and the kernel spectra stream through as whole quads (coalesced float4, two
+// planes of both columns).
 constexpr int kZMixThreads = 128;
 constexpr int kZMixChunk = 32;  // frequency pairs per CTA, one per lane
 
-// Sums of one output plane at frequency k (acc0) and Qy - k (acc1).  Terms
-// whose kernel spectrum is real and those whose spectrum is imaginary are
-// summed apart (r*, i*) and the factor i is applied once at the end, so a
-// term is one load of the spectrum, two shared-memory loads and four FMAs;
-// every parity below is a compile-time constant of the output component A.
-struct ZAcc {
-  float2 r0, r1, i0, i1;
-  __device__ ZAcc() : r0(make_float2(0.f, 0.f)), r1(r0), i0(r0), i1(r0) {}
-  __device__ __forceinline__ void add(bool imag, float v0, float v1, float2 m0, float2 m1) {
-    float2& a0 = imag ? i0 : r0;
-    float2& a1 = imag ? i1 : r1;
-    a0.x = fmaf(v0, m0.x, a0.x); a0.y = fmaf(v0, m0.y, a0.y);
-    a1.x = fmaf(v1, m1.x, a1.x); a1.y = fmaf(v1, m1.y, a1.y);
-  }
-  __device__ __forceinline__ float2 out0() const { return make_float2(r0.x - i0.y, r0.y + i0.x); }
-  __device__ __forceinline__ float2 out1() const { return make_float2(r1.x - i1.y, r1.y + i1.x); }
-};
-
-// H_A(iz) = sum_jz sum_b Ns_Ab(iz - jz) m_b(jz): xz, yz odd in dz and
-// imaginary, xy and yz odd in y (Nq holds dz >= 0)
-template <int A>
-__device__ __forceinline__ ZAcc zmix_demag(const ZMixJob& J, int iz, const float* __restrict__ nq,
-                                           const float2* s0, const float2* s1, size_t kstride) {
-  ZAcc acc;
-  const int nz = J.nz;
-  for (int jz = 0; jz < nz; ++jz) {
-    const int adz = iz >= jz ? iz - jz : jz - iz;
-    const float sz = iz >= jz ? 1.f : -1.f;
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int comp = A == b ? A : (A + b == 1 ? 3 : (A + b == 2 ? 4 : 5));
-      const bool imag = comp >= 4;               // xz, yz
-      const bool odd_y = comp == 3 || comp == 5; // xy, yz
-      const float v = (imag ? sz : 1.f) * __ldg(nq + (size_t)(comp * nz + adz) * kstride);
-      acc.add(imag, v, odd_y ? -v : v, s0[(b * nz + jz) * kZMixChunk], s1[(b * nz + jz) * kZMixChunk]);
-    }
-  }
-  return acc;
-}
-
-// c(o) = sum_jz sum_c T_c(o, jz) m_c(jz), T_x, T_y imaginary, T_y odd in y
-// (A = 2: rows with the parities of S); field variant: H_A(o) with the rows
-// of -N, imaginary when odd in x (xz, zx) or y (yz, zy), odd in y for xy,
-// yx, yz, zy
-template <int A>
-__device__ __forceinline__ ZAcc zmix_coef(const ZMixJob& J, int oc, const float* __restrict__ tq,
-                                          const float2* s0, const float2* s1, size_t kstride) {
-  ZAcc acc;
-  const int nz = J.nz;
-  for (int jz = 0; jz < nz; ++jz) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const bool imag = (A == 2) != (c == 2);
-      const bool odd_y = (A == 1) != (c == 1);
-      const float v = __ldg(tq + (size_t)((oc * nz + jz) * 3 + c) * kstride);
-      acc.add(imag, v, odd_y ? -v : v, s0[(c * nz + jz) * kZMixChunk], s1[(c * nz + jz) * kZMixChunk]);
-    }
-  }
-  return acc;
-}
-
 __global__ void __launch_bounds__(kZMixThreads) k_zmix3(const Launch<ZMixJob> Lc) {
-  extern __shared__ float2 zs[];  // [2][3 nz][kZMixChunk]: inputs at ky, then at Qy - ky
+  extern __shared__ float4 zs[];  // [2][3 nz][kZMixChunk]: inputs at ky, then at Qy - ky with m_y negated
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const ZMixJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
   const int nch = (J.kyq + kZMixChunk - 1) / kZMixChunk;
-  const int kx = tile / nch;
-  const int k0 = (tile - kx * nch) * kZMixChunk;
+  const int kxp = tile / nch;
+  const int k0 = (tile - kxp * nch) * kZMixChunk;
   const int nk = min(kZMixChunk, J.kyq - k0);
+  const int kxa = 2 * kxp;
+  const bool has_b = kxa + 1 < J.kxh;  // an odd last column runs beside itself, stored once
   const int Qy = J.Qy, nz = J.nz, P3 = 3 * nz;
   const size_t pstride = (size_t)J.kxh * Qy;  // one input / output plane
-  const float2* inb = J.in + (size_t)kx * Qy;
+  const int cb = has_b ? Qy : 0;
+  const float2* inb = J.in + (size_t)kxa * Qy;
   for (int i = threadIdx.x; i < P3 * kZMixChunk; i += blockDim.x) {
     const int p = i / kZMixChunk, l = i - p * kZMixChunk;
     if (l < nk) {
       const int k = k0 + l;
-      const bool two = k != 0 && 2 * k != Qy;
+      const int k1 = k != 0 && 2 * k != Qy ? Qy - k : k;
       const float2* row = inb + (size_t)p * pstride;
-      zs[i] = row[k];
-      zs[P3 * kZMixChunk + i] = row[two ? Qy - k : k];
+      const float2 a = row[k], b = row[k + cb];
+      float2 c = row[k1], d = row[k1 + cb];
+      if (p >= nz && p < 2 * nz) {  // odd in y: the sums below then need no sign of their own
+        c.x = -c.x; c.y = -c.y; d.x = -d.x; d.y = -d.y;
+      }
+      zs[i] = make_float4(a.x, b.x, a.y, b.y);
+      zs[P3 * kZMixChunk + i] = make_float4(c.x, d.x, c.y, d.y);
     }
   }
   __syncthreads();
@@ -354,60 +301,133 @@ __global__ void __launch_bounds__(kZMixThreads) k_zmix3(const Launch<ZMixJob> Lc
   if (l >= nk) return;
   const int k = k0 + l;
   const bool two = k != 0 && 2 * k != Qy;
-  const size_t kstride = (size_t)J.kxh * J.kyq;  // one stored kernel plane
-  const size_t koff = (size_t)kx * J.kyq + k;
-  const float2* s0 = zs + l;
-  const float2* s1 = zs + P3 * kZMixChunk + l;
-  const int planes = J.nH + J.n_out;
-  // one output plane per warp at a time (warp-uniform branches below)
-  for (int o = threadIdx.x / kZMixChunk; o < planes; o += kZMixThreads / kZMixChunk) {
-    ZAcc acc;
-    float2* dst;
-    uint16_t* pk;
-    int prow;  // row (plane, kx) of the packed output
-    if (o < J.nH) {
-      const int a = o / nz, iz = o - a * nz;
-      const float* nq = J.Nq + koff;
-      if (a == 0) acc = zmix_demag<0>(J, iz, nq, s0, s1, kstride);
-      else if (a == 1) acc = zmix_demag<1>(J, iz, nq, s0, s1, kstride);
-      else acc = zmix_demag<2>(J, iz, nq, s0, s1, kstride);
-      dst = J.outH + (size_t)o * pstride + (size_t)kx * Qy;
-      pk = J.pkH;
-      prow = o * J.kxh + kx;
-    } else {
-      const int oc = o - J.nH;
-      const int a = J.field_nbox > 0 ? oc / J.field_nbox : 2;  // row z of N has the parities of S
-      const float* tq = J.Tq + koff;
-      if (a == 0) acc = zmix_coef<0>(J, oc, tq, s0, s1, kstride);
-      else if (a == 1) acc = zmix_coef<1>(J, oc, tq, s0, s1, kstride);
-      else acc = zmix_coef<2>(J, oc, tq, s0, s1, kstride);
-      dst = J.outC + (size_t)oc * pstride + (size_t)kx * Qy;
-      pk = J.pkC;
-      prow = oc * J.kxh + kx;
-    }
+  const size_t qs = (size_t)((J.kxh + 1) >> 1) * J.kyq;  // quads of two planes
+  const size_t koff = (size_t)kxp * J.kyq + k;
+  const float4* s0 = zs + l;
+  const float4* s1 = zs + P3 * kZMixChunk + l;
+  const int kch = (Qy + (int)(kKChunk / 2) - 1) / (int)(kKChunk / 2);
+  // value at ky (v0) and at Qy - ky (v1) of plane `o` of an output array
+  auto put = [&](float2* out, uint16_t* pk, int o, bool neg1, c2 v0, c2 v1) {
+    if (neg1) v1 = c2_scale(p2_dup(-1.f), v1);
     if (pk) {  // reduced precision: straight into the inverse DFT's split operand
-      const int kch = (Qy + (int)(kKChunk / 2) - 1) / (int)(kKChunk / 2);
-      store_split(pk, kch, prow, k, acc.out0());
-      if (two) store_split(pk, kch, prow, Qy - k, acc.out1());
+      const int prow = o * J.kxh + kxa;
+      store_split(pk, kch, prow, k, c2_a(v0));
+      if (has_b) store_split(pk, kch, prow + 1, k, c2_b(v0));
+      if (two) {
+        store_split(pk, kch, prow, Qy - k, c2_a(v1));
+        if (has_b) store_split(pk, kch, prow + 1, Qy - k, c2_b(v1));
+      }
+      return;
+    }
+    float2* dst = out + (size_t)o * pstride + (size_t)kxa * Qy;
+    dst[k] = c2_a(v0);
+    if (has_b) dst[k + Qy] = c2_b(v0);
+    if (two) {
+      dst[Qy - k] = c2_a(v1);
+      if (has_b) dst[2 * Qy - k] = c2_b(v1);
+    }
+  };
+  auto in0 = [&](int c, int jz) { return c2_load(s0 + (c * nz + jz) * kZMixChunk); };
+  auto in1 = [&](int c, int jz) { return c2_load(s1 + (c * nz + jz) * kZMixChunk); };
+
+  const int npair = (J.n_out + 1) / 2, ndem = J.nH ? nz : 0;
+  const int ts2 = t_stride(nz, false) / 2;  // quads per coefficient plane
+  for (int task = threadIdx.x / kZMixChunk; task < npair + ndem; task += kZMixThreads / kZMixChunk) {
+    if (task < npair) {
+      // c(o) = sum_jz sum_c T_c(o, jz) m_c(jz), T_x and T_y imaginary (row z of
+      // N too); of the field variant's rows x and y, T_z is the imaginary one
+      const int o = 2 * task;
+      const bool more = o + 1 < J.n_out;
+      const ulonglong2* ta = reinterpret_cast<const ulonglong2*>(J.Tq) + (size_t)o * ts2 * qs + koff;
+      const ulonglong2* tb = more ? ta + (size_t)ts2 * qs : ta;
+      c2 u[2][2], w[2][2];  // [output][side]: the terms of m_x and m_y, those of m_z
+#pragma unroll
+      for (int q = 0; q < 2; ++q)
+#pragma unroll
+        for (int s = 0; s < 2; ++s) u[q][s] = w[q][s] = c2_zero();
+      auto term = [&](int c, int jz, p2 a, p2 b) {
+        const c2 m0 = in0(c, jz), m1 = in1(c, jz);
+        c2(*d)[2] = c == 2 ? w : u;
+        d[0][0] = c2_axpy(a, m0, d[0][0]);
+        d[0][1] = c2_axpy(a, m1, d[0][1]);
+        d[1][0] = c2_axpy(b, m0, d[1][0]);
+        d[1][1] = c2_axpy(b, m1, d[1][1]);
+      };
+      int jz = 0;
+      for (; jz + 1 < nz; jz += 2) {  // two layers: three quads
+        ulonglong2 a[3], b[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+          a[q] = __ldg(ta + q * qs);
+          b[q] = __ldg(tb + q * qs);
+        }
+        ta += 3 * qs;
+        tb += 3 * qs;
+        term(0, jz, a[0].x, b[0].x);
+        term(1, jz, a[0].y, b[0].y);
+        term(2, jz, a[1].x, b[1].x);
+        term(0, jz + 1, a[1].y, b[1].y);
+        term(1, jz + 1, a[2].x, b[2].x);
+        term(2, jz + 1, a[2].y, b[2].y);
+      }
+      if (jz < nz) {
+        const ulonglong2 a0 = __ldg(ta), a1 = __ldg(ta + qs), b0 = __ldg(tb), b1 = __ldg(tb + qs);
+        term(0, jz, a0.x, b0.x);
+        term(1, jz, a0.y, b0.y);
+        term(2, jz, a1.x, b1.x);
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        if (q == 1 && !more) break;
+        const int a = J.field_nbox > 0 ? (o + q) / J.field_nbox : 2;
+        c2 v[2];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) v[s] = a == 2 ? c2_add_i<1>(w[q][s], u[q][s]) : c2_add_i<1>(u[q][s], w[q][s]);
+        put(J.outC, J.pkC, o + q, a == 1, v[0], v[1]);
+      }
     } else {
-      dst[k] = acc.out0();
-      if (two) dst[Qy - k] = acc.out1();
+      // H_a(iz) = sum_jz sum_b Ns_ab(iz - jz) m_b(jz); xz and yz imaginary and odd in dz
+      const int iz = task - npair;
+      c2 r[3][2], i[3][2];
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int s = 0; s < 2; ++s) r[a][s] = i[a][s] = c2_zero();
+      for (int jz = 0; jz < nz; ++jz) {
+        const int adz = iz >= jz ? iz - jz : jz - iz;
+        const ulonglong2* nq = reinterpret_cast<const ulonglong2*>(J.Nq) + (size_t)(3 * adz) * qs + koff;
+        const ulonglong2 q0 = __ldg(nq), q1 = __ldg(nq + qs), q2 = __ldg(nq + 2 * qs);
+        const p2 sz = p2_dup(iz >= jz ? 1.f : -1.f);
+        const p2 xx = q0.x, yy = q0.y, zz = q1.x, xy = q1.y, xz = p2_mul(sz, q2.x), yz = p2_mul(sz, q2.y);
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const c2 mx = s ? in1(0, jz) : in0(0, jz), my = s ? in1(1, jz) : in0(1, jz), mz = s ? in1(2, jz) : in0(2, jz);
+          r[0][s] = c2_axpy(xy, my, c2_axpy(xx, mx, r[0][s]));
+          i[0][s] = c2_axpy(xz, mz, i[0][s]);
+          r[1][s] = c2_axpy(yy, my, c2_axpy(xy, mx, r[1][s]));
+          i[1][s] = c2_axpy(yz, mz, i[1][s]);
+          r[2][s] = c2_axpy(zz, mz, r[2][s]);
+          i[2][s] = c2_axpy(yz, my, c2_axpy(xz, mx, i[2][s]));
+        }
+      }
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        put(J.outH, J.pkH, a * nz + iz, a == 1, c2_add_i<1>(r[a][0], i[a][0]), c2_add_i<1>(r[a][1], i[a][1]));
     }
   }
 }
 
-// CTAs per kx (the output planes are covered inside each CTA)
-int zmix_tiles(int kyq, int planes) {
-  (void)planes;
-  return (kyq + kZMixChunk - 1) / kZMixChunk;
-}
+// CTAs of a job (the output planes are covered inside each)
+int zmix_tiles(int kxh, int kyq) { return (kxh + 1) / 2 * ((kyq + kZMixChunk - 1) / kZMixChunk); }
 
 cudaError_t launch_zmix3(const Launch<ZMixJob>& L, cudaStream_t st) {
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
   int nzmax = 1;
   for (int i = 0; i < L.njobs; ++i) nzmax = max(nzmax, L.job[i].nz);
-  const size_t smem = sizeof(float2) * 2 * 3 * (size_t)nzmax * kZMixChunk;
+  const size_t smem = sizeof(float4) * 2 * 3 * (size_t)nzmax * kZMixChunk;
+  cudaError_t e = cudaFuncSetAttribute(k_zmix3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
   k_zmix3<<<grid, kZMixThreads, smem, st>>>(L);
   return cudaGetLastError();
 }

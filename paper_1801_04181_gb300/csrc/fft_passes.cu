@@ -16,6 +16,7 @@
 // stored values, and walks ky in natural order so those loads coalesce.
 // Thicker magnets (nz > 4) take z by an FFT pass of its own (fft3d.cu).
 #include "fft.cuh"
+#include "fft2.cuh"
 #include "mm_internal.h"
 #include "prefilter.cuh"
 #include "umma.cuh"
@@ -180,13 +181,16 @@ template <int NZ>
 __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int Q, int nH) {
   // output planes per batch of kernel loads (about 30 values in flight)
   constexpr int OB = 30 / (3 * NZ) > 0 ? 30 / (3 * NZ) : 1;
-  const int kstride = J.kxh * J.kyq;  // one stored kernel plane (< 2^31 values in all)
+  // quads (quad_index): plane p of this column at (p / 2) qs + 2 (p % 2)
+  const size_t qs = (size_t)((J.kxh + 1) >> 1) * J.kyq * 4;
+  auto plane = [&](int p) { return (p >> 1) * qs + 2 * (p & 1); };
+  const int ts = t_stride(NZ, true);
   const int half = Q >> 1;
   for (int kyq = threadIdx.x; kyq <= half; kyq += blockDim.x) {
     // the two frequencies ky = kyq and Qy - kyq share every stored kernel value;
     // the second has the odd-in-y components negated
     const bool two = kyq != 0 && 2 * kyq != Q;
-    const int koff = kx * J.kyq + kyq;
+    const size_t koff = 4 * ((size_t)(kx >> 1) * J.kyq + kyq) + (kx & 1);
     const int p0 = fft_pos(kyq, J.fy.plan);
     const int p1 = two ? fft_pos(Q - kyq, J.fy.plan) : p0;
     float2 mh[2][3][NZ];
@@ -201,7 +205,7 @@ __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int
           for (int jz = 0; jz < NZ; ++jz)
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-              tv[o][jz][c] = ob + o < J.n_out ? __ldg(Tk + (((ob + o) * NZ + jz) * 3 + c) * kstride) : 0.f;
+              tv[o][jz][c] = ob + o < J.n_out ? __ldg(Tk + plane((ob + o) * ts + jz * 3 + c)) : 0.f;
         // c(o) = sum_jz sum_c T_c(o, jz) m_c(jz); T = Ms W (S spectra) / (Qx Qy)
 #pragma unroll
         for (int o = 0; o < OB; ++o) {
@@ -229,7 +233,7 @@ __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int
 #pragma unroll
       for (int comp = 0; comp < 6; ++comp)
 #pragma unroll
-        for (int dz = 0; dz < NZ; ++dz) nv[comp][dz] = __ldg(Nk + (comp * NZ + dz) * kstride);
+        for (int dz = 0; dz < NZ; ++dz) nv[comp][dz] = __ldg(Nk + plane(dz * 6 + comp));
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const float fy = side ? -1.f : 1.f;
@@ -262,8 +266,7 @@ __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int
 // warps) covers the 271 frequency pairs of a 540-point line in one round of
 // the spectral products.
 constexpr int kYThreads = 288;
-// FIX540: every job's y plan is 540 = 4 9 15, run with its lengths as constants.
-template <int NZ, unsigned RSET, bool FIX540>
+template <int NZ, unsigned RSET>
 __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Launch<YJob> Lc) {
   constexpr int Pin = 3 * NZ;
   extern __shared__ float2 sm[];
@@ -277,20 +280,6 @@ __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Laun
   const int ny = J.ny;
   const float2* col0 = J.in + (size_t)kx * ny;
   const size_t pstride = (size_t)J.kxh * ny;  // one input plane
-
-  // The kernel spectra of this kx column are read only after the forward FFT:
-  // start moving their lines into L2 now (one prefetch per 128-byte line).
-  {
-    const size_t kstride = (size_t)J.kxh * J.kyq;
-    const int lines = (J.kyq + 31) / 32;
-    const int nN = J.do_H ? 6 * NZ : 0;
-    const int nT = J.do_C ? 3 * NZ * J.n_out : 0;
-    for (int i = threadIdx.x; i < (nN + nT) * lines; i += blockDim.x) {
-      const int row = i / lines, ln = i - row * lines;
-      const float* p = row < nN ? J.Nq + (size_t)row * kstride : J.Tq + (size_t)(row - nN) * kstride;
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(p + (size_t)kx * J.kyq + 32 * ln));
-    }
-  }
 
   if ((ny & 1) == 0) {
     // one float4 (two complex rows) of every plane per thread and step
@@ -321,12 +310,10 @@ __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Laun
   if (J.do_C)
     build_pref_table(tab, J.r + 2 * kPrefWarm + kYChunk, J.box_lo, J.box_len, J.start, Q, nullptr, J.periodic != 0);
   __syncthreads();
-  if constexpr (FIX540) fft_smem_fixed<kFwdDif, float2, 4, 9, 15>(sm, Pin, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
-  else fft_smem<kFwdDif, float2, RSET>(sm, Q, Pin, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+  fft_smem<kFwdDif, float2, RSET>(sm, Q, Pin, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
   ypass_mix<NZ>(J, sm, kx, Q, nH);
   __syncthreads();
-  if constexpr (FIX540) fft_smem_fixed<kInvDit, float2, 4, 9, 15>(sm, Pout, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
-  else fft_smem<kInvDit, float2, RSET>(sm, Q, Pout, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+  fft_smem<kInvDit, float2, RSET>(sm, Q, Pout, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
 
   if (J.do_H) {
     float2* out0 = J.outH + (size_t)kx * ny;
@@ -355,6 +342,229 @@ __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Laun
         for (int o = 0; o < J.n_out; ++o) out0[o * ostride + k] = sm[(nH + o) * Q + t];
       }
     }
+  }
+}
+
+// ------------------------------------------------------------------ y pass, two columns per CTA
+// The same pass on the columns kx and kx + 1 as one pair of lines per plane
+// (fft2.cuh): transforms, spectral products and the prefilter run both columns
+// in packed arithmetic.
+
+// Spectral products of the coefficient planes [c0, c1) (placed from plane cb
+// on) and, last, of the demag planes, at every (ky, Qy - ky) pair.  Terms whose
+// kernel spectrum is real and those whose spectrum is imaginary are summed
+// apart and the factor i is applied once; at Qy - ky the components odd in y
+// change sign, which is the same as negating m_y there and H_y in the result.
+// One thread per frequency of a pair (neighbouring lanes: their loads
+// coincide); the kernel values come as quads, both columns packed.
+template <int NZ>
+__device__ __forceinline__ void ypass2_mix(const YJob& J, float4* sm, int kxp, int Q, int cb, int c0, int c1,
+                                           bool do_H) {
+  constexpr int TS = t_stride(NZ, true);
+  constexpr int OB = NZ == 1 ? 4 : NZ == 2 ? 3 : 1;  // outputs per batch of loads: whole quads
+  constexpr int TQ = (OB * TS + 1) / 2;    // their quads
+  const unsigned qs = (unsigned)((J.kxh + 1) >> 1) * J.kyq;  // quads of two planes
+  const p2 minus = p2_dup(-1.f);
+  for (int item = threadIdx.x; item < 2 * J.kyq; item += blockDim.x) {
+    const int kyq = item >> 1;
+    const bool mirror = (item & 1) != 0;  // this thread's frequency is Qy - kyq
+    if (mirror && (kyq == 0 || 2 * kyq == Q)) continue;
+    float4* at = sm + __ldg(J.fy.pos + (mirror ? Q - kyq : kyq));
+    c2 mh[3][NZ];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int z = 0; z < NZ; ++z) mh[c][z] = c2_load(at + (c * NZ + z) * Q);
+    if (mirror)
+#pragma unroll
+      for (int z = 0; z < NZ; ++z) mh[1][z] = c2_scale(minus, mh[1][z]);
+    const unsigned koff = (unsigned)kxp * J.kyq + kyq;
+    const ulonglong2* Tk = reinterpret_cast<const ulonglong2*>(J.Tq) + koff;
+    for (int ob = c0; ob < c1; ob += OB) {
+      p2 tv[2 * TQ];
+#pragma unroll
+      for (int q = 0; q < TQ; ++q) {
+        // quads of outputs past the last are not read (a batch starts on a whole quad)
+        if (ob + (2 * q) / TS < c1) {
+          const ulonglong2 v = __ldg(Tk + (size_t)(ob * TS / 2 + q) * qs);
+          tv[2 * q] = v.x; tv[2 * q + 1] = v.y;
+        } else {
+          tv[2 * q] = tv[2 * q + 1] = 0ull;
+        }
+      }
+      // c(o) = sum_jz sum_c T_c(o, jz) m_c(jz); T_x, T_y imaginary, T_z real
+#pragma unroll
+      for (int o = 0; o < OB; ++o) {
+        if (ob + o >= c1) break;
+        const p2* t = tv + o * TS;
+        c2 r = c2_scale(t[2], mh[2][0]), i = c2_scale(t[0], mh[0][0]);
+        i = c2_axpy(t[1], mh[1][0], i);
+#pragma unroll
+        for (int jz = 1; jz < NZ; ++jz) {
+          r = c2_axpy(t[3 * jz + 2], mh[2][jz], r);
+          i = c2_axpy(t[3 * jz], mh[0][jz], i);
+          i = c2_axpy(t[3 * jz + 1], mh[1][jz], i);
+        }
+        c2_store(at + (cb + ob + o - c0) * Q, c2_add_i<1>(r, i));
+      }
+    }
+    if (!do_H) continue;
+    // H_a(iz) = sum_jz sum_b Ns_ab(iz - jz) m_b(jz), the planes dz * 6 + (xx yy
+    // zz xy xz yz); xz and yz imaginary and odd in dz
+    const ulonglong2* Nk = reinterpret_cast<const ulonglong2*>(J.Nq) + koff;
+    p2 nv[6 * NZ];
+#pragma unroll
+    for (int q = 0; q < 3 * NZ; ++q) {
+      const ulonglong2 v = __ldg(Nk + (size_t)q * qs);
+      nv[2 * q] = v.x; nv[2 * q + 1] = v.y;
+    }
+#pragma unroll
+    for (int iz = 0; iz < NZ; ++iz) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        c2 r = c2_zero(), ip = r, im = r;  // real terms; imaginary ones with dz >= 0 and dz < 0
+#pragma unroll
+        for (int jz = 0; jz < NZ; ++jz) {
+          const int adz = iz >= jz ? iz - jz : jz - iz;
+#pragma unroll
+          for (int b = 0; b < 3; ++b) {
+            const int comp = a == b ? a : a + b + 2;
+            const bool imag = (a == 2) != (b == 2);
+            if (!imag) r = c2_axpy(nv[adz * 6 + comp], mh[b][jz], r);
+            else if (iz >= jz) ip = c2_axpy(nv[adz * 6 + comp], mh[b][jz], ip);
+            else im = c2_axpy(nv[adz * 6 + comp], mh[b][jz], im);
+          }
+        }
+        c2 h = c2_add_i<1>(r, iz + 1 < NZ ? ip - im : ip);  // no dz < 0 term in the last layer
+        if (a == 1 && mirror) h = c2_scale(minus, h);
+        c2_store(at + (a * NZ + iz) * Q, h);
+      }
+    }
+  }
+}
+
+// Planes of a CTA in shared memory: the 3 NZ input planes (then the demag
+// planes, in place) and `ch` coefficient planes at a time.
+//
+// What bounds it: shared memory and the latency of the kernel spectra between
+// the barriers (stick-slip films: 46% of the shared-memory wavefronts, 37%
+// issue-active, 17% DRAM).  Against the one-column pass, 45 M warp instructions
+// for 64 M and 94 -> 92 us there; one 1024 x 1024 film over another (one CTA
+// per SM in both) 411 -> 322 us, 355 x 145 x 3 over 301 x 127 x 2 37 + 26 -> 26 +
+// 23 us, 64 x 64 x 1 19 -> 13 us.  640 or 512 threads per SM (fewer, with more
+// registers) measured 0-10% slower over these sizes.
+constexpr int kY2Threads = 768;  // per SM, shared out over its CTAs
+template <int NZ, typename Fft>
+__global__ void __launch_bounds__(kY2Threads, 1) k_ypass2(const Launch<YJob> Lc) {
+  constexpr int Pin = 3 * NZ;
+  extern __shared__ float4 sm4[];
+  const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
+  const YJob& J = Lc.job[j];
+  const int kxa = 2 * (blockIdx.x - Lc.tile_start[j]);
+  const bool has_b = kxa + 1 < J.kxh;  // an odd last column runs beside itself, stored once
+  const int Q = Fft::kL ? Fft::kL : J.fy.plan.L;
+  const int n_out = J.do_C ? J.n_out : 0;
+  const int ch = J.ch;
+  const int cb = J.do_H || ch < n_out ? Pin : 0;  // alone and at once, the coefficient planes go in place
+  float4* tws = sm4 + max(Pin, cb + ch) * Q;
+  int* tab = reinterpret_cast<int*>(tws + J.fy.ntw2);
+  const int ny = J.ny;
+  const size_t pstride = (size_t)J.kxh * ny;  // one input plane
+
+  {
+    // rows [ny, Q) are zero padding; column b follows column a
+    const float2* ca = J.in + (size_t)kxa * ny;
+    const int nb = has_b ? ny : 0;
+    Fft::template in<kFwdDif>(
+        sm4, Q, Pin, J.fy, tws,
+        [&](int p, int y0, int M, auto& v) {
+          const float2* src = ca + p * pstride + y0;
+#pragma unroll
+          for (int k = 0; k < (int)(sizeof(v) / sizeof(v[0])); ++k)
+            v[k] = y0 + k * M < ny ? c2_make(__ldg(src + k * M), __ldg(src + k * M + nb)) : c2_zero();
+        },
+        [&]() {
+          for (int i = threadIdx.x; i < J.fy.ntw2; i += blockDim.x) tws[i] = __ldg(J.fy.tw2 + i);
+          if (n_out)
+            build_pref_table(tab, J.r + 2 * kPrefWarm + kYChunk, J.box_lo, J.box_len, J.start, Q, nullptr,
+                             J.periodic != 0);
+          // The kernel spectra of these columns are read after the forward FFT:
+          // start moving their lines into L2 (one prefetch per 128-byte line).
+          const size_t qs = (size_t)((J.kxh + 1) >> 1) * J.kyq;
+          const int lines = (J.kyq + 7) / 8;  // eight quads
+          const int nN = J.do_H ? 3 * NZ : 0, nT = (t_stride(NZ, true) * n_out + 1) / 2;
+          for (int row = threadIdx.x / 32; row < nN + nT; row += blockDim.x / 32) {
+            const float4* p = reinterpret_cast<const float4*>(row < nN ? J.Nq : J.Tq) +
+                              (row < nN ? row : row - nN) * qs + (size_t)(kxa >> 1) * J.kyq;
+            for (int ln = threadIdx.x % 32; ln < lines; ln += 32)
+              asm volatile("prefetch.global.L2 [%0];" ::"l"(p + 8 * ln));
+          }
+        });
+  }
+  for (int c0 = 0;; c0 += ch) {
+    const int c1 = min(c0 + ch, n_out);
+    const bool last = c1 >= n_out;
+    const bool H = last && J.do_H;
+    ypass2_mix<NZ>(J, sm4, kxa >> 1, Q, cb, c0, c1, H);
+    __syncthreads();
+    // inverse of the demag planes (rows y < ny straight to memory) with the
+    // last coefficient planes, which follow them
+    float4* first = H ? sm4 : sm4 + cb * Q;
+    const int nh = H ? Pin : 0, lines = nh + c1 - c0;
+    float2* oa = J.outH + (size_t)kxa * ny;
+    Fft::out(first, Q, lines, J.fy, tws, [&](int p, int y0, int M, auto& v) {
+      constexpr int R = (int)(sizeof(v) / sizeof(v[0]));
+      if (p >= nh) {
+        float4* dst = first + p * Q + y0;
+#pragma unroll
+        for (int k = 0; k < R; ++k) c2_store(dst + k * M, v[k]);
+      } else {
+        float2* dst = oa + p * pstride + y0;
+#pragma unroll
+        for (int k = 0; k < R; ++k)
+          if (y0 + k * M < ny) {
+            dst[k * M] = c2_a(v[k]);
+            if (has_b) dst[k * M + ny] = c2_b(v[k]);
+          }
+      }
+    });
+    // y prefilter and the coefficient rows
+    const int r = J.r, ncol = c1 - c0;
+    float2* oc = J.outC + ((size_t)c0 * J.kxh + kxa) * r;
+    const size_t ostride = (size_t)J.kxh * r;
+    const float4* col0 = first + nh * Q;
+    if (J.fir) {
+      // one thread per chunk and per real or imaginary part (of both columns);
+      // the two parts swap halves to store whole values
+      const int nch = (r + kYChunk - 1) / kYChunk;
+      const int items = 2 * ncol * nch;
+      for (int base = threadIdx.x & ~31; base < items; base += blockDim.x) {
+        const int at = base + (int)(threadIdx.x & 31), idx = min(at, items - 1);  // whole warps swap (items is even)
+        const int o = (idx >> 1) / nch, part = idx & 1;
+        const int k0 = ((idx >> 1) - o * nch) * kYChunk;
+        const p2* src = reinterpret_cast<const p2*>(col0 + o * Q) + part;
+        float2* dst = oc + o * ostride + part * r;
+        const bool store = (part == 0 || has_b) && at < items;
+        prefilter_chunk2<kYChunk>(
+            k0, [&](int jj) { return src[2 * tab[jj]]; },
+            [&](int k, p2 v) {
+              const float2 f = p2_unpack(v);  // (column a, column b) of this part
+              const float other = __shfl_xor_sync(0xffffffffu, part ? f.x : f.y, 1);
+              if (store && k < r) dst[k] = part ? make_float2(other, f.y) : make_float2(f.x, other);
+            });
+      }
+    } else {
+      for (int k = threadIdx.x; ncol > 0 && k < r; k += blockDim.x) {
+        const int t = tab[k + kPrefWarm];
+        for (int o = 0; o < ncol; ++o) {
+          const float4 v = col0[o * Q + t];
+          oc[o * ostride + k] = make_float2(v.x, v.z);
+          if (has_b) oc[o * ostride + k + r] = make_float2(v.y, v.w);
+        }
+      }
+    }
+    if (last) break;
+    __syncthreads();  // the next planes overwrite these
   }
 }
 
@@ -512,22 +722,86 @@ cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-template <int NZ>
-static cudaError_t launch_ypass_nz(const Launch<YJob>& L, size_t smem, cudaStream_t st) {
-  unsigned rs = 0;
-  bool fix540 = true;
-  for (int i = 0; i < L.njobs; ++i) {
-    rs |= plan_radix_set(L.job[i].fy.plan);
-    fix540 = fix540 && fixed_plan_id(L.job[i].fy.plan) == 3;
+// The y pass of jobs of one layer count, two columns per CTA where their lines
+// fit shared memory.
+constexpr size_t kSmemMax = 227 * 1024;              // per CTA
+constexpr size_t kSmemTwo = (228 * 1024) / 2 - 1024;  // each of two CTAs on an SM
+
+// the pair plans with builds of their own (0: none)
+static int pair_plan_id(const FftPlanDev& P) {
+  static const int plans[][5] = {{3, 4, 8, 5, 0}, {3, 4, 8, 9, 0}, {3, 12, 9, 5, 0}, {3, 12, 9, 10, 0}, {4, 6, 8, 9, 5}};
+  for (int i = 0; i < 5; ++i) {
+    bool same = P.nstages == plans[i][0];
+    for (int s = 0; same && s < P.nstages; ++s) same = P.radix[s] == plans[i][1 + s];
+    if (same) return i + 1;
   }
-  auto k = fix540 ? k_ypass<NZ, kRadixSetA, true>
-                  : (rs & ~kRadixSetA) == 0u ? k_ypass<NZ, kRadixSetA, false> : k_ypass<NZ, kAllRadices, false>;
+  return 0;
+}
+
+static size_t ypass2_smem(const YJob& J, int ch) {
+  const int n_out = J.do_C ? J.n_out : 0;
+  const int cb = J.do_H || ch < n_out ? 3 * J.nz : 0;
+  return ((size_t)max(3 * J.nz, cb + ch) * J.fy.plan.L + J.fy.ntw2) * sizeof(float4) +
+         ypass_table_bytes(n_out ? J.r : 0);
+}
+
+// Coefficient planes at a time: all of them, or the most that let two CTAs
+// share an SM, or the most that fit; 0 if that is none.  Chunks start on whole
+// quads of the kernel spectra: one layer's hold two planes.
+static int ypass2_chunk(const YJob& J) {
+  const int n_out = J.do_C ? J.n_out : 0;
+  for (size_t limit : {kSmemTwo, kSmemMax}) {
+    if (ypass2_smem(J, n_out) <= limit) return max(n_out, 1);
+    for (int ch = n_out - 1; ch >= 1; --ch)
+      if (ypass2_smem(J, ch) <= limit && (J.nz > 1 || ch % 2 == 0)) return ch;
+  }
+  return 0;
+}
+
+template <int NZ>
+static cudaError_t launch_ypass_nz(const Launch<YJob>& L0, size_t smem1, cudaStream_t st) {
+  Launch<YJob> L = L0;
+  unsigned rs = 0;
+  bool pairs = true;
+  int id = -1;
+  size_t smem = 0;
+  for (int i = 0; i < L.njobs; ++i) {
+    YJob& J = L.job[i];
+    rs |= plan_radix_set(J.fy.plan);
+    J.ch = ypass2_chunk(J);
+    id = id < 0 || id == pair_plan_id(J.fy.plan) ? pair_plan_id(J.fy.plan) : 0;
+    pairs = pairs && J.ch > 0;
+    smem = max(smem, ypass2_smem(J, J.ch));
+  }
+  void (*k)(const Launch<YJob>);
+  int threads = kYThreads;
+  if (pairs) {
+    // the lengths of 64, 128, 256, 512 and 1024 cells (4 cells of margin) with
+    // their plans as constants, 13% faster at 540; else the plan at run time
+    k = id == 1   ? k_ypass2<NZ, CtPair<4, 8, 5>>
+        : id == 2 ? k_ypass2<NZ, CtPair<4, 8, 9>>
+        : id == 3 ? k_ypass2<NZ, CtPair<12, 9, 5>>
+        : id == 4 ? k_ypass2<NZ, CtPair<12, 9, 10>>
+        : id == 5 ? k_ypass2<NZ, CtPair<6, 8, 9, 5>>
+        : (rs & ~kRadixSetB) == 0u ? k_ypass2<NZ, RtPair<kRadixSetB>> : k_ypass2<NZ, RtPair<kAllRadices>>;
+    const int ctas = min(3, max(1, (int)(228 * 1024 / (smem + 1024))));
+    threads = kY2Threads / ctas / 32 * 32;
+    int tiles = 0;
+    for (int i = 0; i < L.njobs; ++i) {
+      L.tile_start[i] = tiles;
+      tiles += (L.job[i].kxh + 1) / 2;
+    }
+    L.tile_start[L.njobs] = tiles;
+  } else {
+    k = (rs & ~kRadixSetA) == 0u ? k_ypass<NZ, kRadixSetA> : k_ypass<NZ, kAllRadices>;
+    smem = smem1;
+  }
   max_carveout((const void*)k);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, kYThreads, smem, st>>>(L);
+  k<<<grid, threads, smem, st>>>(L);
   return cudaGetLastError();
 }
 

@@ -282,9 +282,11 @@ __global__ void k_extract_quarter(const double2* spec, double* out, int Qx, int 
   out[(size_t)kx * kyq + ky] = take_imag ? v.y : v.x;
 }
 
-// T[o][jz][c] = scale * sum_zb W[o][zb] Sq[(zb - jz) - dz_lo][c]  (quarter planes)
+// T[o][jz][c] = scale * sum_zb W[o][zb] Sq[(zb - jz) - dz_lo][c]  (quarter
+// planes), stored as quads, plane o * tstride + jz * 3 + c
 __global__ void k_mix_T(const double* Sq, const double* W, float* T, int n_out, int nz, int bz,
-                        int dz_first_plane_offset, size_t qsize, double scale) {
+                        int dz_first_plane_offset, int kxh, int kyq, int tstride, double scale) {
+  const size_t qsize = (size_t)kxh * kyq;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= qsize) return;
   const int c = blockIdx.y;
@@ -297,14 +299,16 @@ __global__ void k_mix_T(const double* Sq, const double* W, float* T, int n_out, 
     const int plane = zb - jz + dz_first_plane_offset;
     acc += w * Sq[((size_t)plane * 3 + c) * qsize + i];
   }
-  T[((size_t)oj * 3 + c) * qsize + i] = (float)(scale * acc);
+  T[quad_index(o * tstride + jz * 3 + c, (int)(i / kyq), (int)(i % kyq), kxh, kyq)] = (float)(scale * acc);
 }
 
 // Componentwise field variant: TN[(a n_out + o) nz + jz][b] = scale * sum_zb
 // W[o][zb] N_ab((zb - jz) - dz_lo), from the six N components of every z
-// offset (Nq6 [plane][6][qsize], xx yy zz xy xz yz).
+// offset (Nq6 [plane][6][qsize], xx yy zz xy xz yz); quads, plane
+// (a n_out + o) tstride + jz * 3 + b.
 __global__ void k_mix_TN(const double* Nq6, const double* W, float* T, int n_out, int nz, int bz,
-                         size_t qsize, double scale) {
+                         int kxh, int kyq, int tstride, double scale) {
+  const size_t qsize = (size_t)kxh * kyq;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= qsize) return;
   const int a = blockIdx.y / 3, b = blockIdx.y - 3 * (blockIdx.y / 3);
@@ -318,7 +322,15 @@ __global__ void k_mix_TN(const double* Nq6, const double* W, float* T, int n_out
     const int plane = zb - jz + nz - 1;
     acc += w * Nq6[((size_t)plane * 6 + comp) * qsize + i];
   }
-  T[((((size_t)a * n_out + o) * nz + jz) * 3 + b) * qsize + i] = (float)(scale * acc);
+  T[quad_index((a * n_out + o) * tstride + jz * 3 + b, (int)(i / kyq), (int)(i % kyq), kxh, kyq)] =
+      (float)(scale * acc);
+}
+
+// one quarter plane into plane `plane` of a quad array
+__global__ void k_put_quads(const double* in, float* out, int plane, int kxh, int kyq, double scale) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i < (size_t)kxh * kyq)
+    out[quad_index(plane, (int)(i / kyq), (int)(i % kyq), kxh, kyq)] = (float)(scale * in[i]);
 }
 
 __global__ void k_scale_to_float(const double* in, float* out, size_t n, double scale) {
@@ -375,12 +387,8 @@ cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftT
   for (int dz = 0; dz < K.nz; ++dz) {
     cudaError_t e = plane_spectra(1, 6, K, dz, a, b, c, fx, fy, work, qbuf, imag6, st);
     if (e != cudaSuccess) return e;
-    // Nq layout [6][nz][kxh][kyq]
-    for (int q = 0; q < 6; ++q) {
-      const size_t n = qsize;
-      k_scale_to_float<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(
-          qbuf + q * qsize, Nq + ((size_t)q * K.nz + dz) * qsize, n, scale);
-    }
+    for (int q = 0; q < 6; ++q)
+      k_put_quads<<<(unsigned)((qsize + 255) / 256), 256, 0, st>>>(qbuf + q * qsize, Nq, dz * 6 + q, kxh, kyq, scale);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -389,7 +397,7 @@ cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftT
 
 cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                             double b, double c, double scale, int box_lo_z, int bz, int n_out,
-                            const double* W_dev, float* Tq, double2* work, double* Sq,
+                            const double* W_dev, float* Tq, int tstride, double2* work, double* Sq,
                             cudaStream_t st) {
   const int kxh = K.Qx / 2 + 1, kyq = K.Qy / 2 + 1;
   const size_t qsize = (size_t)kxh * kyq;
@@ -403,7 +411,7 @@ cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftT
   }
   // plane index of offset dz = (box_lo_z + zb) - jz is (zb - jz) + (nz - 1)
   dim3 g((unsigned)((qsize + 255) / 256), 3, n_out * K.nz);
-  k_mix_T<<<g, 256, 0, st>>>(Sq, W_dev, Tq, n_out, K.nz, bz, K.nz - 1, qsize, scale);
+  k_mix_T<<<g, 256, 0, st>>>(Sq, W_dev, Tq, n_out, K.nz, bz, K.nz - 1, kxh, kyq, tstride, scale);
   return cudaGetLastError();
 }
 
@@ -420,7 +428,8 @@ cudaError_t build_TN_spectra(const KernelPlan& K, const FftTables& fx, const Fft
     if (e != cudaSuccess) return e;
   }
   dim3 g((unsigned)((qsize + 255) / 256), 9, n_out * K.nz);
-  k_mix_TN<<<g, 256, 0, st>>>(Nq6, W_dev, TN, n_out, K.nz, bz, qsize, scale);
+  k_mix_TN<<<g, 256, 0, st>>>(Nq6, W_dev, TN, n_out, K.nz, bz, K.Qx / 2 + 1, K.Qy / 2 + 1, t_stride(K.nz, false),
+                              scale);
   return cudaGetLastError();
 }
 

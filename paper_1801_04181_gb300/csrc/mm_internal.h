@@ -21,6 +21,7 @@ constexpr unsigned kAllRadices = 2047u;
 // the set the FFT pass kernels are also built for: {4, 9, 15, 16} (every length
 // 4^a 9^b 15^c 16^d, among them 540 = 4 9 15 and 2160 = 16 9 15)
 constexpr unsigned kRadixSetA = 4u | 64u | 512u | 1024u;
+constexpr unsigned kRadixSetB = kAllRadices & ~(512u | 1024u);
 
 struct FftPlanDev {
   int L;
@@ -37,6 +38,21 @@ struct FftPlanDev {
   int stw_off[kMaxStages];
 };
 
+// Kernel spectra of the direct z sums, in quads: the values of two planes at
+// two neighbouring kx columns are adjacent (plane p col a, p col b, p + 1 col a,
+// p + 1 col b), so a thread that takes both columns loads two planes' packed
+// pairs as one coalesced float4.  Quads of [plane / 2][kx / 2][ky].
+__host__ __device__ inline size_t quad_index(int plane, int kx, int ky, int kxh, int kyq) {
+  return ((((size_t)(plane >> 1) * ((kxh + 1) >> 1) + (kx >> 1)) * kyq + ky) << 2) | ((plane & 1) << 1) | (kx & 1);
+}
+__host__ __device__ inline size_t quad_floats(int planes, int kxh, int kyq) {
+  return (size_t)((planes + 1) >> 1) * ((kxh + 1) >> 1) * kyq * 4;
+}
+// planes of N: dz * 6 + component; planes of T: o * stride + jz * 3 + c, the
+// stride even (whole quads per output) except for the fused pass on one layer,
+// which takes two outputs at a time
+__host__ __device__ constexpr int t_stride(int nz, bool fused) { return fused && nz == 1 ? 3 : (3 * nz + 1) & ~1; }
+
 // Length-L transform resources resident on the device.
 struct FftTables {
   FftPlanDev plan;
@@ -44,6 +60,11 @@ struct FftTables {
   const double2* tw_d;
   const int* pos;         // frequency k -> position in DIF output
   const int* freq;        // position -> frequency
+  // pair table (fft2.cuh): stage s from entry tw2_off[s], row n1 < M of
+  // (c, c, s, s) of W_Lb^{n1 k}, k = 1 .. R-1 (pitch odd); the last stage has none
+  const float4* tw2;
+  int tw2_off[kMaxStages];
+  int ntw2;
 };
 
 // ---------------------------------------------------------------- x forward
@@ -66,15 +87,16 @@ struct YJob {
   int kyq;                // Qy/2 + 1 stored ky values of the kernel spectra
   // self-demag output
   int do_H;
-  const float* Nq;        // [6][nz][kxh][kyq]  (xx yy zz xy xz yz; dz >= 0)
+  const float* Nq;        // quads, planes dz * 6 + (xx yy zz xy xz yz), dz >= 0
   float2* outH;           // [3 nz][kxh][ny]
   // potential / coefficient output
   int do_C;
   int n_out;
-  const float* Tq;        // [n_out][nz][3][kxh][kyq]
+  const float* Tq;        // quads, planes o * t_stride(nz, true) + jz * 3 + c
   float2* outC;           // [n_out][kxh][r]
   int box_lo, box_len, start, r, fir;
   int periodic;           // the y box is the whole period: the prefilter wraps
+  int ch;                 // coefficient planes held at once (set by launch_ypass)
 };
 
 // ---------------------------------------------------------------- x inverse
@@ -135,8 +157,8 @@ struct YInvJob {
 struct ZMixJob {
   const float2* in;       // [3 nz][kxh][Qy]
   int nz, kxh, Qy, kyq;
-  const float* Nq;        // [6][nz][kxh][kyq]
-  const float* Tq;        // [n_out][nz][3][kxh][kyq]
+  const float* Nq;        // quads, planes dz * 6 + component
+  const float* Tq;        // quads, planes o * t_stride(nz, false) + jz * 3 + c
   int nH, n_out;          // output planes: 3 nz demag (if nH), then n_out coefficient planes
   float2* outH;           // [3 nz][kxh][Qy]
   float2* outC;           // [n_out][kxh][Qy]
@@ -399,7 +421,7 @@ size_t divcurl_cells(int nx, int ny, int nz);
 int divcurl_blocks(int nx, int ny, int nz);
 cudaError_t launch_divcurl(const float* H, int nx, int ny, int nz, double dx, double dy, double dz,
                            double* partial, double* out, cudaStream_t st);
-int zmix_tiles(int kyq, int planes);
+int zmix_tiles(int kxh, int kyq);
 int zpass_tile(int Qz);                 // y positions per z-pass CTA for a z grid
 int zpass_tiles(int Qy, int ztile);
 int gather_tiles(int nx, int ny, int nz);  // 32 x 8 columns x up to kMaxNz layers
@@ -413,7 +435,7 @@ cudaError_t eval_points_fp64(int kind, int n, const double* off_dev, double a, d
                              double* out_dev, cudaStream_t st);
 cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                             double b, double c, double scale, float* Nq, double2* work, double* qbuf,
-                            cudaStream_t st);
+                            cudaStream_t st);  // quads (quad_index)
 // 3D spectra of S (kind 0, 3 comps) or N (kind 1, 6 comps): out [comp][kxh][kyq][kzq].
 // Scratch: work 2 * ncomp * Qx * Qy double2, q2 ncomp * Qz * kxh * kyq double,
 // qtmp ncomp * kxh * kyq double, zl kxh * kyq * Qz double2.
@@ -428,13 +450,13 @@ cudaError_t build_spectra_3d(int kind, const KernelPlan3& K, const FftTables& fx
 // doubles, work as for build_N_spectra.
 cudaError_t build_TN_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                              double b, double c, double scale, int box_lo_z, int bz, int n_out,
-                             const double* W_dev, float* TN, double2* work, double* Nq6, cudaStream_t st);
+                             const double* W_dev, float* TN, double2* work, double* Nq6, cudaStream_t st);  // quads
 cudaError_t build_S_planes(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a, double b,
                            double c, double scale, int dz_lo, int nplanes, float* Sq, double2* work,
                            double* qtmp, cudaStream_t st);
 cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                             double b, double c, double scale, int box_lo_z, int bz, int n_out,
-                            const double* W_dev, float* Tq, double2* work, double* Sq,
-                            cudaStream_t st);
+                            const double* W_dev, float* Tq, int tstride, double2* work, double* Sq,
+                            cudaStream_t st);  // quads
 
 }  // namespace mm

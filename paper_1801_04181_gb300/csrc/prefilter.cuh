@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "fft.cuh"
+#include "fft2.cuh"
 
 namespace mm {
 
@@ -56,6 +57,26 @@ __device__ __forceinline__ void prefilter_chunk(int k0, int r, Src src, Out out)
   for (int i = CH + kPrefWarm - 1; i >= 0; --i) {
     c = ybuf[i] + kZ1 * c;
     if (i < CH && k0 + i < r) out(k0 + i, kPrefGain * c);
+  }
+}
+
+// prefilter_chunk on one part (real or imaginary) of a pair of lines, packed;
+// out is called for every k of the chunk, by all threads alike.
+template <int CH, typename Src, typename Out>
+__device__ __forceinline__ void prefilter_chunk2(int k0, Src src, Out out) {
+  const p2 z = p2_dup(kZ1), g = p2_dup(kPrefGain);
+  p2 ybuf[CH + kPrefWarm];
+  p2 y = 0ull;
+#pragma unroll
+  for (int j = 0; j < CH + 2 * kPrefWarm; ++j) {
+    y = p2_fma(z, y, src(k0 + j));
+    if (j >= kPrefWarm) ybuf[j - kPrefWarm] = y;
+  }
+  p2 c = 0ull;
+#pragma unroll
+  for (int i = CH + kPrefWarm - 1; i >= 0; --i) {
+    c = p2_fma(z, c, ybuf[i]);
+    if (i < CH) out(k0 + i, p2_mul(g, c));
   }
 }
 
