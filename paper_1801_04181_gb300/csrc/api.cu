@@ -2512,7 +2512,7 @@ static mm_status eddy_core(mm_ctx* ctx, int mag, const float* dBdt_dev, double s
   int sweeps = 0;
   double stats[3] = {0, 0, 0};
   for (;;) {
-    CK(launch_sor_residual(M.ed_phi, M.ed_b, M.ed_stats + 3, M.nx, M.ny, M.nz, M.d, M.ed_part, M.ed_stats, st));
+    CK(launch_sor_residual(M.ed_phi, M.ed_b, M.nx, M.ny, M.nz, M.d, M.ed_part, M.ed_stats, st));
     CK(cudaMemcpyAsync(stats, M.ed_stats, sizeof(stats), cudaMemcpyDeviceToHost, st));
     CK(cudaStreamSynchronize(st));
     if (stats[0] <= kTol * stats[1] || stats[1] == 0.0) break;
@@ -2520,7 +2520,7 @@ static mm_status eddy_core(mm_ctx* ctx, int mag, const float* dBdt_dev, double s
       if (sweeps_out) *sweeps_out = sweeps;
       return fail(ctx, MM_ETIMEOUT, "mm_eddy_field: the electric potential did not converge");
     }
-    CK(launch_sor_sweeps(M.ed_phi, M.ed_b, M.ed_stats + 3, M.nx, M.ny, M.nz, M.d, omega, kCheck, st));
+    CK(launch_sor_sweeps(M.ed_phi, M.ed_b, M.nx, M.ny, M.nz, M.d, omega, kCheck, st));
     sweeps += kCheck;
   }
   if (sweeps_out) *sweeps_out = sweeps;

@@ -103,32 +103,77 @@ __global__ void __launch_bounds__(256) k_sum_parts(const double* __restrict__ pa
   if (threadIdx.x == 0) *out = scale * red[0];
 }
 
-// one colour of a red-black SOR sweep: cells with (x + y + z) % 2 == colour
-__global__ void __launch_bounds__(256) k_sor(double* __restrict__ phi, const double* __restrict__ b,
-                                             const double* __restrict__ bmean, int nx, int ny, int nz, double wx,
-                                             double wy, double wz, double omega, int colour) {
-  const size_t N = (size_t)nx * ny * nz;
+// the source with its mean removed, in place
+__global__ void __launch_bounds__(256) k_sub_mean(double* __restrict__ b, size_t N, const double* __restrict__ mean) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const CellIdx c = cell_of(i, nx, ny);
-  if (((c.x + c.y + c.z) & 1) != colour) return;
-  double s = 0.0, w = 0.0;
-  if (c.x > 0) { s += wx * phi[i - 1]; w += wx; }
-  if (c.x < nx - 1) { s += wx * phi[i + 1]; w += wx; }
-  if (c.y > 0) { s += wy * phi[i - nx]; w += wy; }
-  if (c.y < ny - 1) { s += wy * phi[i + nx]; w += wy; }
-  if (c.z > 0) { s += wz * phi[i - (size_t)nx * ny]; w += wz; }
-  if (c.z < nz - 1) { s += wz * phi[i + (size_t)nx * ny]; w += wz; }
-  if (w == 0.0) return;  // a single cell: phi = 0
-  const double gs = (s - (b[i] - *bmean)) / w;
-  phi[i] += omega * (gs - phi[i]);
+  if (i < N) b[i] -= *mean;
+}
+
+// Weights of the SOR update: w per axis, and c = omega / (sum of the weights of
+// the neighbours present), by the number of neighbours along each axis.
+struct SorCoef {
+  double wx, wy, wz, omega1;  // omega1 = 1 - omega
+  double c[27];               // [present x + 3 present y + 9 present z]
+};
+
+// One colour of a red-black SOR sweep, cells with (x + y + z) % 2 == colour, a
+// thread per cell of the colour: phi <- (1 - omega) phi + c (sum w phi_nb - b').
+// The FP64 pipe is what bounds it (two operations per clock and SM): nine
+// operations a cell, no division (the sum, the weights and the quotient written
+// out per neighbour were about 35: 30 us a colour at 64^3, now 4 us).
+__global__ void __launch_bounds__(256) k_sor(double* __restrict__ phi, const double* __restrict__ b, int nx, int ny,
+                                             int nz, const SorCoef C, int colour) {
+  const unsigned nh = (unsigned)(nx + 1) >> 1;  // cells of a colour per row, at most
+  const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
+  const unsigned row = i / nh;
+  if (row >= (unsigned)ny * (unsigned)nz) return;
+  const int z = (int)(row / (unsigned)ny), y = (int)(row - (unsigned)z * (unsigned)ny);
+  const int x = 2 * (int)(i - row * nh) + ((y + z + colour) & 1);
+  if (x >= nx) return;
+  const size_t p = (size_t)row * nx + x, sz = (size_t)nx * ny;
+  const bool xm = x > 0, xp = x < nx - 1, ym = y > 0, yp = y < ny - 1, zm = z > 0, zp = z < nz - 1;
+  const int present = (xm + xp) + 3 * (ym + yp) + 9 * (zm + zp);
+  if (present == 0) return;  // a single cell: phi = 0
+  const double sx = (xm ? phi[p - 1] : 0.0) + (xp ? phi[p + 1] : 0.0);
+  const double sy = (ym ? phi[p - nx] : 0.0) + (yp ? phi[p + nx] : 0.0);
+  const double s_z = (zm ? phi[p - sz] : 0.0) + (zp ? phi[p + sz] : 0.0);
+  const double t = fma(C.wx, sx, fma(C.wy, sy, fma(C.wz, s_z, -b[p])));
+  phi[p] = fma(C.c[present], t, C.omega1 * phi[p]);
+}
+
+// Non-negative doubles compare like their bit patterns (the integer pipe, not
+// the FP64 one); a NaN counts as zero, as fmax has it.
+__device__ __forceinline__ unsigned long long max_bits(double v) {
+  return v > 0.0 ? (unsigned long long)__double_as_longlong(v) : 0ull;
+}
+__device__ __forceinline__ unsigned long long umax64(unsigned long long a, unsigned long long b) { return a > b ? a : b; }
+
+// block maxima of r and bb and the block sum of p, in thread 0, in a fixed order
+__device__ __forceinline__ void residual_reduce(unsigned long long& r, unsigned long long& bb, double& p) {
+  __shared__ unsigned long long rs[8], bs[8];
+  __shared__ double ps[8];
+  for (int o = 16; o > 0; o >>= 1) {
+    r = umax64(r, __shfl_down_sync(0xffffffffu, r, o));
+    bb = umax64(bb, __shfl_down_sync(0xffffffffu, bb, o));
+    p += __shfl_down_sync(0xffffffffu, p, o);
+  }
+  const int w = threadIdx.x >> 5;
+  if ((threadIdx.x & 31) == 0) {
+    rs[w] = r; bs[w] = bb; ps[w] = p;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int k = 1; k < 8; ++k) {
+      r = umax64(r, rs[k]);
+      bb = umax64(bb, bs[k]);
+      p += ps[k];
+    }
 }
 
 // per-block max |A phi - b'| and max |b'|, and the block sum of phi (its mean)
 __global__ void __launch_bounds__(256) k_sor_residual(const double* __restrict__ phi, const double* __restrict__ b,
-                                                      const double* __restrict__ bmean, int nx, int ny, int nz,
-                                                      double wx, double wy, double wz, double* __restrict__ part) {
-  __shared__ double rmax[256], bmax[256], psum[256];
+                                                      int nx, int ny, int nz, double wx, double wy, double wz,
+                                                      double* __restrict__ part) {
   const size_t N = (size_t)nx * ny * nz;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   double r = 0.0, bb = 0.0, p = 0.0;
@@ -142,56 +187,34 @@ __global__ void __launch_bounds__(256) k_sor_residual(const double* __restrict__
     if (c.y < ny - 1) s += wy * (phi[i + nx] - f);
     if (c.z > 0) s += wz * (phi[i - (size_t)nx * ny] - f);
     if (c.z < nz - 1) s += wz * (phi[i + (size_t)nx * ny] - f);
-    const double bi = b[i] - *bmean;
-    r = fabs(s - bi);
-    bb = fabs(bi);
+    r = fabs(s - b[i]);
+    bb = fabs(b[i]);
     p = f;
   }
-  rmax[threadIdx.x] = r;
-  bmax[threadIdx.x] = bb;
-  psum[threadIdx.x] = p;
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      rmax[threadIdx.x] = fmax(rmax[threadIdx.x], rmax[threadIdx.x + s]);
-      bmax[threadIdx.x] = fmax(bmax[threadIdx.x], bmax[threadIdx.x + s]);
-      psum[threadIdx.x] += psum[threadIdx.x + s];
-    }
-    __syncthreads();
-  }
+  unsigned long long rb = max_bits(r), bbb = max_bits(bb);
+  residual_reduce(rb, bbb, p);
   if (threadIdx.x == 0) {
-    part[3 * blockIdx.x] = rmax[0];
-    part[3 * blockIdx.x + 1] = bmax[0];
-    part[3 * blockIdx.x + 2] = psum[0];
+    part[3 * blockIdx.x] = __longlong_as_double((long long)rb);
+    part[3 * blockIdx.x + 1] = __longlong_as_double((long long)bbb);
+    part[3 * blockIdx.x + 2] = p;
   }
 }
 
 // out[0] = max residual, out[1] = max |b'|, out[2] = mean phi (one block)
 __global__ void __launch_bounds__(256) k_residual_reduce(const double* __restrict__ part, int nparts, double invN,
                                                          double* __restrict__ out) {
-  __shared__ double rmax[256], bmax[256], psum[256];
-  double r = 0.0, bb = 0.0, p = 0.0;
+  unsigned long long r = 0ull, bb = 0ull;
+  double p = 0.0;
   for (int k = threadIdx.x; k < nparts; k += blockDim.x) {
-    r = fmax(r, part[3 * k]);
-    bb = fmax(bb, part[3 * k + 1]);
+    r = umax64(r, max_bits(part[3 * k]));
+    bb = umax64(bb, max_bits(part[3 * k + 1]));
     p += part[3 * k + 2];
   }
-  rmax[threadIdx.x] = r;
-  bmax[threadIdx.x] = bb;
-  psum[threadIdx.x] = p;
-  __syncthreads();
-  for (int s = 128; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      rmax[threadIdx.x] = fmax(rmax[threadIdx.x], rmax[threadIdx.x + s]);
-      bmax[threadIdx.x] = fmax(bmax[threadIdx.x], bmax[threadIdx.x + s]);
-      psum[threadIdx.x] += psum[threadIdx.x + s];
-    }
-    __syncthreads();
-  }
+  residual_reduce(r, bb, p);
   if (threadIdx.x == 0) {
-    out[0] = rmax[0];
-    out[1] = bmax[0];
-    out[2] = psum[0] * invN;
+    out[0] = __longlong_as_double((long long)r);
+    out[1] = __longlong_as_double((long long)bb);
+    out[2] = p * invN;
   }
 }
 
@@ -272,24 +295,32 @@ cudaError_t launch_eddy_source(const float* E, int nx, int ny, int nz, const dou
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_sum_parts<<<1, 256, 0, st>>>(part, (int)blocks(N), 1.0 / (double)N, bmean);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_sub_mean<<<blocks(N), 256, 0, st>>>(b, N, bmean);
   return cudaGetLastError();
 }
 
-cudaError_t launch_sor_sweeps(double* phi, const double* b, const double* bmean, int nx, int ny, int nz,
-                              const double d[3], double omega, int sweeps, cudaStream_t st) {
-  const size_t N = (size_t)nx * ny * nz;
-  const double wx = 1.0 / (d[0] * d[0]), wy = 1.0 / (d[1] * d[1]), wz = 1.0 / (d[2] * d[2]);
+cudaError_t launch_sor_sweeps(double* phi, const double* b, int nx, int ny, int nz, const double d[3], double omega,
+                              int sweeps, cudaStream_t st) {
+  SorCoef C;
+  C.wx = 1.0 / (d[0] * d[0]); C.wy = 1.0 / (d[1] * d[1]); C.wz = 1.0 / (d[2] * d[2]);
+  C.omega1 = 1.0 - omega;
+  for (int k = 0; k < 27; ++k) {
+    const double w = (k % 3) * C.wx + (k / 3 % 3) * C.wy + (k / 9) * C.wz;
+    C.c[k] = w > 0.0 ? omega / w : 0.0;
+  }
+  const size_t n = (size_t)((nx + 1) / 2) * ny * nz;
   for (int k = 0; k < sweeps; ++k)
-    for (int colour = 0; colour < 2; ++colour)
-      k_sor<<<blocks(N), 256, 0, st>>>(phi, b, bmean, nx, ny, nz, wx, wy, wz, omega, colour);
+    for (int colour = 0; colour < 2; ++colour) k_sor<<<blocks(n), 256, 0, st>>>(phi, b, nx, ny, nz, C, colour);
   return cudaGetLastError();
 }
 
-cudaError_t launch_sor_residual(const double* phi, const double* b, const double* bmean, int nx, int ny, int nz,
-                                const double d[3], double* part, double* stats, cudaStream_t st) {
+cudaError_t launch_sor_residual(const double* phi, const double* b, int nx, int ny, int nz, const double d[3],
+                                double* part, double* stats, cudaStream_t st) {
   const size_t N = (size_t)nx * ny * nz;
   const double wx = 1.0 / (d[0] * d[0]), wy = 1.0 / (d[1] * d[1]), wz = 1.0 / (d[2] * d[2]);
-  k_sor_residual<<<blocks(N), 256, 0, st>>>(phi, b, bmean, nx, ny, nz, wx, wy, wz, part);
+  k_sor_residual<<<blocks(N), 256, 0, st>>>(phi, b, nx, ny, nz, wx, wy, wz, part);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k_residual_reduce<<<1, 256, 0, st>>>(part, (int)blocks(N), 1.0 / (double)N, stats);

@@ -398,10 +398,10 @@ cudaError_t launch_accumulate(const float* in, size_t N, float* out, cudaStream_
 int eddy_blocks(size_t N);
 cudaError_t launch_eddy_source(const float* E, int nx, int ny, int nz, const double d[3], double* b, double* part,
                                double* bmean, cudaStream_t st);
-cudaError_t launch_sor_sweeps(double* phi, const double* b, const double* bmean, int nx, int ny, int nz,
-                              const double d[3], double omega, int sweeps, cudaStream_t st);
-cudaError_t launch_sor_residual(const double* phi, const double* b, const double* bmean, int nx, int ny, int nz,
-                                const double d[3], double* part, double* stats, cudaStream_t st);
+cudaError_t launch_sor_sweeps(double* phi, const double* b, int nx, int ny, int nz, const double d[3], double omega,
+                              int sweeps, cudaStream_t st);
+cudaError_t launch_sor_residual(const double* phi, const double* b, int nx, int ny, int nz, const double d[3],
+                                double* part, double* stats, cudaStream_t st);
 cudaError_t launch_eddy_current(const double* phi, const double* stats, const float* E, int nx, int ny, int nz,
                                 const double d[3], double sigma, float* J, cudaStream_t st);
 cudaError_t launch_flux_rate(const float* Hself, const float* Hstray, const float* y, size_t N, const double hext[3],
