@@ -259,6 +259,23 @@ static mm_status eddy_core(mm_ctx* ctx, int mag, const float* dBdt_dev, double s
                            int* sweeps_out);
 static mm_status cross_eddy_field(mm_ctx* ctx, int g, const float* J, float* H);
 
+namespace mm {
+cudaError_t allow_smem(const void* kernel, size_t dynamic_max) {
+  static std::mutex mu;
+  static std::set<std::pair<int, const void*>> done;  // (device, kernel): a few dozen at most per device
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  if (done.count({dev, kernel})) return cudaSuccess;
+  e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dynamic_max);
+  if (e == cudaSuccess) done.insert({dev, kernel});
+  return e;
+}
+}  // namespace mm
+
 // ============================================================ helpers
 namespace {
 

@@ -120,12 +120,13 @@ struct SorCoef {
 // thread per cell of the colour: phi <- (1 - omega) phi + c (sum w phi_nb - b').
 // The FP64 pipe is what bounds it (two operations per clock and SM): nine
 // operations a cell, no division (the sum, the weights and the quotient written
-// out per neighbour were about 35: 30 us a colour at 64^3, now 4 us).
+// out per neighbour were about 35: 18 us a colour at 64^3, now 6 us).
 __global__ void __launch_bounds__(256) k_sor(double* __restrict__ phi, const double* __restrict__ b, int nx, int ny,
                                              int nz, const SorCoef C, int colour) {
   const unsigned nh = (unsigned)(nx + 1) >> 1;  // cells of a colour per row, at most
   const unsigned i = blockIdx.x * blockDim.x + threadIdx.x;
   const unsigned row = i / nh;
+  pdl_wait();
   if (row >= (unsigned)ny * (unsigned)nz) return;
   const int z = (int)(row / (unsigned)ny), y = (int)(row - (unsigned)z * (unsigned)ny);
   const int x = 2 * (int)(i - row * nh) + ((y + z + colour) & 1);
@@ -312,8 +313,11 @@ cudaError_t launch_sor_sweeps(double* phi, const double* b, int nx, int ny, int 
   }
   const size_t n = (size_t)((nx + 1) / 2) * ny * nz;
   for (int k = 0; k < sweeps; ++k)
-    for (int colour = 0; colour < 2; ++colour) k_sor<<<blocks(n), 256, 0, st>>>(phi, b, nx, ny, nz, C, colour);
-  return cudaGetLastError();
+    for (int colour = 0; colour < 2; ++colour) {
+      cudaError_t e = launch_chained(k_sor, blocks(n), 256, 0, st, phi, b, nx, ny, nz, C, colour);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
 
 cudaError_t launch_sor_residual(const double* phi, const double* b, int nx, int ny, int nz, const double d[3],

@@ -40,6 +40,7 @@ cudaError_t init_fft_constants_3d() { return upload_roots(); }
 template <unsigned RSET, int FIXP>
 __global__ void __launch_bounds__(256, 3) k_yfwd3(const Launch<YFwdJob> Lc) {
   extern __shared__ float2 sm[];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const YFwdJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
@@ -80,6 +81,7 @@ __device__ __forceinline__ float2 c_i_times(float2 m) { return make_float2(-m.y,
 template <unsigned RSET>
 __global__ void __launch_bounds__(256, 2) k_zpass3(const Launch<ZJob> Lc) {
   extern __shared__ float2 sm[];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const ZJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
@@ -192,6 +194,7 @@ __global__ void __launch_bounds__(256, 2) k_zpass3(const Launch<ZJob> Lc) {
 template <unsigned RSET, int FIXP>
 __global__ void __launch_bounds__(256, 3) k_yinv3(const Launch<YInvJob> Lc) {
   extern __shared__ float2 sm[];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const YInvJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
@@ -248,12 +251,6 @@ __global__ void __launch_bounds__(256, 3) k_yinv3(const Launch<YInvJob> Lc) {
   }
 }
 
-// dynamic shared memory of a launch, with the carveout set to shared memory
-static cudaError_t prep(const void* f, size_t smem) {
-  cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-}
-
 // ------------------------------------------------------------------ direct z sum
 // The plane mixing of Sec. III.A for sources of up to kMaxNzDirect layers.
 // CTA -> (two kx columns, a chunk of kZMixChunk frequency pairs ky, Qy - ky):
@@ -268,6 +265,7 @@ constexpr int kZMixChunk = 32;  // frequency pairs per CTA, one per lane
 
 __global__ void __launch_bounds__(kZMixThreads) k_zmix3(const Launch<ZMixJob> Lc) {
   extern __shared__ float4 zs[];  // [2][3 nz][kZMixChunk]: inputs at ky, then at Qy - ky with m_y negated
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const ZMixJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
@@ -426,10 +424,7 @@ cudaError_t launch_zmix3(const Launch<ZMixJob>& L, cudaStream_t st) {
   int nzmax = 1;
   for (int i = 0; i < L.njobs; ++i) nzmax = max(nzmax, L.job[i].nz);
   const size_t smem = sizeof(float4) * 2 * 3 * (size_t)nzmax * kZMixChunk;
-  cudaError_t e = cudaFuncSetAttribute(k_zmix3, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_zmix3<<<grid, kZMixThreads, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k_zmix3, grid, kZMixThreads, smem, st, L);
 }
 
 // ------------------------------------------------------------------ host side
@@ -453,12 +448,11 @@ cudaError_t launch_yfwd3(const Launch<YFwdJob>& L, cudaStream_t st) {
   for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set(L.job[i].fy.plan);
   auto k = y_fixed_1080(L) ? k_yfwd3<kAllRadices, 2>
            : (rs & ~kRadixSetA) == 0u ? k_yfwd3<kRadixSetA, 0> : k_yfwd3<kAllRadices, 0>;
-  cudaError_t e = prep((const void*)k, smem);
+  cudaError_t e = allow_smem((const void*)k, 227 * 1024);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, 256, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k, grid, 256, smem, st, L);
 }
 
 cudaError_t launch_zpass3(const Launch<ZJob>& L, cudaStream_t st) {
@@ -472,12 +466,11 @@ cudaError_t launch_zpass3(const Launch<ZJob>& L, cudaStream_t st) {
   unsigned rs = 0;
   for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set(L.job[i].fz.plan);
   auto k = (rs & ~kRadixSetA) == 0u ? k_zpass3<kRadixSetA> : k_zpass3<kAllRadices>;
-  cudaError_t e = prep((const void*)k, smem);
+  cudaError_t e = allow_smem((const void*)k, 227 * 1024);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, 256, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k, grid, 256, smem, st, L);
 }
 
 cudaError_t launch_yinv3(const Launch<YInvJob>& L, cudaStream_t st) {
@@ -492,12 +485,11 @@ cudaError_t launch_yinv3(const Launch<YInvJob>& L, cudaStream_t st) {
   for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set(L.job[i].fy.plan);
   auto k = y_fixed_1080(L) ? k_yinv3<kAllRadices, 2>
            : (rs & ~kRadixSetA) == 0u ? k_yinv3<kRadixSetA, 0> : k_yinv3<kAllRadices, 0>;
-  cudaError_t e = prep((const void*)k, smem);
+  cudaError_t e = allow_smem((const void*)k, 227 * 1024);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, 256, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k, grid, 256, smem, st, L);
 }
 
 }  // namespace mm

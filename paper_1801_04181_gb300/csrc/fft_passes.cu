@@ -36,6 +36,7 @@ cudaError_t init_fft_constants_passes() { return upload_roots(); }
 template <unsigned RSET, int FIXP>
 __global__ void __launch_bounds__(kXFwdThreads, 3) k_xfwd(const Launch<XFwdJob> Lc) {
   extern __shared__ float2 sm[];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const XFwdJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
@@ -270,6 +271,7 @@ template <int NZ, unsigned RSET>
 __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Launch<YJob> Lc) {
   constexpr int Pin = 3 * NZ;
   extern __shared__ float2 sm[];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const YJob& J = Lc.job[j];
   const int kx = blockIdx.x - Lc.tile_start[j];
@@ -458,6 +460,7 @@ template <int NZ, typename Fft>
 __global__ void __launch_bounds__(kY2Threads, 1) k_ypass2(const Launch<YJob> Lc) {
   constexpr int Pin = 3 * NZ;
   extern __shared__ float4 sm4[];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const YJob& J = Lc.job[j];
   const int kxa = 2 * (blockIdx.x - Lc.tile_start[j]);
@@ -578,6 +581,7 @@ __device__ __forceinline__ void xinv_put(float2* sm, int off, int Q, int kx, flo
 template <unsigned RSET, int FIXP>
 __global__ void __launch_bounds__(kXInvThreads, 3) k_xinv(const Launch<XInvJob> Lc) {
   extern __shared__ float2 sm[];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const XInvJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
@@ -700,9 +704,7 @@ template <typename JobT> static int x_fixed_plan(const Launch<JobT>& L) {
   return id;
 }
 
-static void max_carveout(const void* f) {
-  cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-}
+constexpr size_t kSmemMax = 227 * 1024;              // per CTA
 
 cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st) {
   const size_t smem =
@@ -713,18 +715,15 @@ cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st) {
   auto k = fx == 1 ? k_xfwd<kRadixSetA, 1>
            : fx == 2 ? k_xfwd<kAllRadices, 2>
            : (rs & ~kRadixSetA) == 0u ? k_xfwd<kRadixSetA, 0> : k_xfwd<kAllRadices, 0>;
-  max_carveout((const void*)k);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k, kSmemMax);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, kXFwdThreads, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k, grid, kXFwdThreads, smem, st, L);
 }
 
 // The y pass of jobs of one layer count, two columns per CTA where their lines
 // fit shared memory.
-constexpr size_t kSmemMax = 227 * 1024;              // per CTA
 constexpr size_t kSmemTwo = (228 * 1024) / 2 - 1024;  // each of two CTAs on an SM
 
 // the pair plans with builds of their own (0: none)
@@ -796,13 +795,11 @@ static cudaError_t launch_ypass_nz(const Launch<YJob>& L0, size_t smem1, cudaStr
     k = (rs & ~kRadixSetA) == 0u ? k_ypass<NZ, kRadixSetA> : k_ypass<NZ, kAllRadices>;
     smem = smem1;
   }
-  max_carveout((const void*)k);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k, kSmemMax);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, threads, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k, grid, threads, smem, st, L);
 }
 
 // Jobs of different layer counts go to separate launches of the matching kernel.
@@ -838,13 +835,11 @@ cudaError_t launch_xinv(const Launch<XInvJob>& L, int Qmax, cudaStream_t st) {
   auto k = fx == 1 ? k_xinv<kRadixSetA, 1>
            : fx == 2 ? k_xinv<kAllRadices, 2>
            : (rs & ~kRadixSetA) == 0u ? k_xinv<kRadixSetA, 0> : k_xinv<kAllRadices, 0>;
-  max_carveout((const void*)k);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k, kSmemMax);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, kXInvThreads, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k, grid, kXInvThreads, smem, st, L);
 }
 
 }  // namespace mm

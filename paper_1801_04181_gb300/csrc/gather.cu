@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(TX * TY, 4) k_gather(const Launch<GatherJob> L
   extern __shared__ float gsm[];
   __shared__ float w_s[3][12];
   __shared__ float red_s[TX * TY / 32][4];
+  pdl_wait();
 
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const GatherJob& J = Lc.job[j];
@@ -243,14 +244,11 @@ cudaError_t launch_gather(const Launch<GatherJob>& L, int nz_max, cudaStream_t s
   bool wrap = false;
   for (int i = 0; i < L.njobs; ++i) wrap = wrap || L.job[i].wrapP[0] > 0 || L.job[i].wrapP[1] > 0;
   auto k = wrap ? k_gather<true> : k_gather<false>;
-  cudaFuncSetAttribute((const void*)k, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       cudaSharedmemCarveoutMaxShared);
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)k, 96 * 1024);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k<<<grid, TX * TY, smem, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k, grid, TX * TY, smem, st, L);
 }
 
 }  // namespace mm

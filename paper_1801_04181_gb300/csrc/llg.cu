@@ -33,6 +33,7 @@ __device__ __forceinline__ float warp_max(float v) {
 template <bool WRAP, bool EDDY, int SG>
 __global__ void __launch_bounds__(256, 6) k_stage(const Launch<StageJob> Lc, const MechParams Perr, int* ticket) {
   __shared__ float red[8];
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const StageJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(256, 6) k_stage(const Launch<StageJob> Lc, con
 
 // y_next = y + sum_j comb[j] k_j   (stage input built from stored k only)
 __global__ void __launch_bounds__(256) k_combine(const Launch<CombineJob> Lc) {
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const CombineJob& J = Lc.job[j];
   const size_t i = (size_t)(blockIdx.x - Lc.tile_start[j]) * blockDim.x + threadIdx.x;
@@ -177,6 +179,7 @@ __global__ void __launch_bounds__(256) k_combine(const Launch<CombineJob> Lc) {
 
 // y = normalise(src)  (accepted step)
 __global__ void __launch_bounds__(256) k_normalise(const Launch<CombineJob> Lc) {
+  pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const CombineJob& J = Lc.job[j];
   const size_t i = (size_t)(blockIdx.x - Lc.tile_start[j]) * blockDim.x + threadIdx.x;
@@ -186,7 +189,10 @@ __global__ void __launch_bounds__(256) k_normalise(const Launch<CombineJob> Lc) 
   J.out[i] = a * inv; J.out[J.n + i] = b * inv; J.out[2 * J.n + i] = c * inv;
 }
 
-__global__ void __launch_bounds__(256) k_mech(const MechParams P) { mech_block(P); }
+__global__ void __launch_bounds__(256) k_mech(const MechParams P) {
+  pdl_wait();
+  mech_block(P);
+}
 
 cudaError_t launch_stage(const Launch<StageJob>& L, const MechParams& Perr, int* ticket, cudaStream_t st) {
   const int grid = L.tile_start[L.njobs];
@@ -203,36 +209,32 @@ cudaError_t launch_stage(const Launch<StageJob>& L, const MechParams& Perr, int*
     if (L.job[i].mode != 0 || L.job[i].stage != sg) sg = 0;
   if (wrap || eddy) sg = 0;
   switch (sg) {
-    case 1: k_stage<false, false, 1><<<grid, 256, 0, st>>>(L, Perr, ticket); break;
-    case 2: k_stage<false, false, 2><<<grid, 256, 0, st>>>(L, Perr, ticket); break;
-    case 3: k_stage<false, false, 3><<<grid, 256, 0, st>>>(L, Perr, ticket); break;
-    case 4: k_stage<false, false, 4><<<grid, 256, 0, st>>>(L, Perr, ticket); break;
-    case 5: k_stage<false, false, 5><<<grid, 256, 0, st>>>(L, Perr, ticket); break;
-    case 6: k_stage<false, false, 6><<<grid, 256, 0, st>>>(L, Perr, ticket); break;
-    case 7: k_stage<false, false, 7><<<grid, 256, 0, st>>>(L, Perr, ticket); break;
+    case 1: return launch_chained(k_stage<false, false, 1>, grid, 256, 0, st, L, Perr, ticket);
+    case 2: return launch_chained(k_stage<false, false, 2>, grid, 256, 0, st, L, Perr, ticket);
+    case 3: return launch_chained(k_stage<false, false, 3>, grid, 256, 0, st, L, Perr, ticket);
+    case 4: return launch_chained(k_stage<false, false, 4>, grid, 256, 0, st, L, Perr, ticket);
+    case 5: return launch_chained(k_stage<false, false, 5>, grid, 256, 0, st, L, Perr, ticket);
+    case 6: return launch_chained(k_stage<false, false, 6>, grid, 256, 0, st, L, Perr, ticket);
+    case 7: return launch_chained(k_stage<false, false, 7>, grid, 256, 0, st, L, Perr, ticket);
     default:
-      if (wrap && eddy) k_stage<true, true, 0><<<grid, 256, 0, st>>>(L, Perr, ticket);
-      else if (wrap) k_stage<true, false, 0><<<grid, 256, 0, st>>>(L, Perr, ticket);
-      else if (eddy) k_stage<false, true, 0><<<grid, 256, 0, st>>>(L, Perr, ticket);
-      else k_stage<false, false, 0><<<grid, 256, 0, st>>>(L, Perr, ticket);
+      if (wrap && eddy) return launch_chained(k_stage<true, true, 0>, grid, 256, 0, st, L, Perr, ticket);
+      else if (wrap) return launch_chained(k_stage<true, false, 0>, grid, 256, 0, st, L, Perr, ticket);
+      else if (eddy) return launch_chained(k_stage<false, true, 0>, grid, 256, 0, st, L, Perr, ticket);
+      else return launch_chained(k_stage<false, false, 0>, grid, 256, 0, st, L, Perr, ticket);
   }
-  return cudaGetLastError();
 }
 cudaError_t launch_combine(const Launch<CombineJob>& L, cudaStream_t st) {
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k_combine<<<grid, 256, 0, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k_combine, grid, 256, 0, st, L);
 }
 cudaError_t launch_normalise(const Launch<CombineJob>& L, cudaStream_t st) {
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  k_normalise<<<grid, 256, 0, st>>>(L);
-  return cudaGetLastError();
+  return launch_chained(k_normalise, grid, 256, 0, st, L);
 }
 cudaError_t launch_mech(const MechParams& P, cudaStream_t st) {
-  k_mech<<<1, 256, 0, st>>>(P);
-  return cudaGetLastError();
+  return launch_chained(k_mech, 1, 256, 0, st, P);
 }
 
 }  // namespace mm
