@@ -35,6 +35,38 @@ namespace mm {
 // this translation unit's copy of the small-DFT roots (see fft.cuh)
 cudaError_t init_fft_constants_3d() { return upload_roots(); }
 
+// The block's lines from memory: f(l, i) loads point i < n of line l < nl, and
+// sm[l ldl + i] takes it, kLineBatch loads of a thread in flight (one at a time,
+// a short line waited out the memory latency once per line).
+constexpr int kLineBatch = 8;
+template <typename Ld>
+__device__ __forceinline__ void load_lines(float2* sm, int ldl, int nl, int n, Ld f) {
+  // a warp takes 32 consecutive points of a line at a time
+  const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int per = (n + 31) >> 5, runs = nl * per;
+  for (int r0 = warp; r0 < runs; r0 += kLineBatch * warps) {
+    float2 v[kLineBatch];
+    int l = r0 / per, c = r0 - l * per;  // line and run of the line, walked without divisions
+    const int l0 = l, c0 = c;
+#pragma unroll
+    for (int u = 0; u < kLineBatch; ++u) {
+      const int i = (c << 5) + lane;
+      if (l < nl && i < n) v[u] = f(l, i);
+      c += warps;
+      while (c >= per) { c -= per; ++l; }
+    }
+    l = l0;
+    c = c0;
+#pragma unroll
+    for (int u = 0; u < kLineBatch; ++u) {
+      const int i = (c << 5) + lane;
+      if (l < nl && i < n) sm[l * ldl + i] = v[u];
+      c += warps;
+      while (c >= per) { c -= per; ++l; }
+    }
+  }
+}
+
 // ------------------------------------------------------------------ y forward
 // FIXP > 0: every job's y plan is fixed plan FIXP, run with its lengths as constants.
 template <unsigned RSET, int FIXP>
@@ -50,16 +82,16 @@ __global__ void __launch_bounds__(256, 3) k_yfwd3(const Launch<YFwdJob> Lc) {
   const int np = min(J.group, J.planes - p0);
   const int Q = FIXP ? FixedPlan<FIXP ? FIXP : 1>::L : J.fy.plan.L;
   const int ldl = Q + 1;  // odd stride: the plane-fastest reads below spread over the banks
-  for (int l = 0; l < np; ++l) {
-    const float2* col = J.in + ((size_t)(p0 + l) * J.kxh + kx) * J.ny;
-    for (int y = threadIdx.x; y < Q; y += blockDim.x)
-      sm[l * ldl + y] = y < J.ny ? col[y] : make_float2(0.f, 0.f);
-  }
+  const int ny = J.ny;
+  const float2* in0 = J.in + ((size_t)p0 * J.kxh + kx) * ny;
+  const size_t pstride = (size_t)J.kxh * ny;
+  load_lines(sm, ldl, np, ny, [&](int l, int y) { return in0[l * pstride + y]; });
   __syncthreads();
+  // rows [ny, Q) are zero padding: the first stage takes them as zero unread
   if constexpr (FIXP > 0)
-    fft_smem_plan<kFwdDif, FIXP, FixedPlan<FIXP>::L + 1>(sm, np, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+    fft_smem_plan<kFwdDif, FIXP, FixedPlan<FIXP>::L + 1>(sm, np, J.fy.plan, J.fy.tw_f, 0, blockDim.x, ny);
   else
-    fft_smem<kFwdDif, float2, RSET>(sm, ldl, np, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+    fft_smem<kFwdDif, float2, RSET>(sm, ldl, np, J.fy.plan, J.fy.tw_f, 0, blockDim.x, ny);
   if (J.natural) {
     // frequency ky read from its DIF position: whole contiguous output rows
     for (int l = 0; l < np; ++l) {
@@ -69,6 +101,10 @@ __global__ void __launch_bounds__(256, 3) k_yfwd3(const Launch<YFwdJob> Lc) {
     return;
   }
   float2* dst = J.out + (size_t)kx * Q * J.planes + p0;
+  if (np == 16) {
+    for (int i = threadIdx.x; i < 16 * Q; i += blockDim.x) dst[(size_t)(i >> 4) * J.planes + (i & 15)] = sm[(i & 15) * ldl + (i >> 4)];
+    return;
+  }
   for (int i = threadIdx.x; i < Q * np; i += blockDim.x) {
     const int p = i / np, l = i - p * np;
     dst[(size_t)p * J.planes + l] = sm[l * ldl + p];
@@ -87,74 +123,67 @@ __global__ void __launch_bounds__(256, 2) k_zpass3(const Launch<ZJob> Lc) {
   const int tile = blockIdx.x - Lc.tile_start[j];
   const int Qy = J.fy.plan.L, Qz = J.fz.plan.L;
   const int zt = J.ztile;
-  const int npt = (Qy + zt - 1) / zt;
+  const int zl = 31 - __clz(zt);  // zt is a power of two
+  const int npt = (Qy + zt - 1) >> zl;
   const int kx = tile / npt;
-  const int y0 = (tile - kx * npt) * zt;
+  const int y0 = (tile - kx * npt) << zl;
   const int nt = min(zt, Qy - y0);
   const int nz = J.nz, P3 = 3 * nz;
   const int ldz = Qz + 1;
   // lines: t * 3 + c (input, then H in place) for t < nt; phi line t at 3 zt + t
   float2* phi = sm + 3 * zt * ldz;
   int* tab = reinterpret_cast<int*>(sm + 4 * zt * ldz);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
 
+  // the 3 nz values of a y position are one run in memory, nz of each component
   const float2* src = J.in + ((size_t)kx * Qy + y0) * P3;
-  for (int i = threadIdx.x; i < nt * P3; i += blockDim.x) {
-    const int t = i / P3, q = i - t * P3;
-    const int c = q / nz, z = q - c * nz;
-    sm[(t * 3 + c) * ldz + z] = src[i];
-  }
-  const int pad = Qz - nz;
-  for (int i = threadIdx.x; i < nt * 3 * pad; i += blockDim.x) {
-    const int l = i / pad, z = nz + (i - l * pad);
-    sm[l * ldz + z] = make_float2(0.f, 0.f);
-  }
+  load_lines(sm, ldz, 3 * nt, nz, [&](int l, int z) { return src[(size_t)l * nz + z]; });
   if (J.do_C) build_pref_table(tab, J.r + 2 * kPrefWarm + kZChunk, J.box_lo, J.box_len, J.start, Qz, nullptr);
   __syncthreads();
-  fft_smem<kFwdDif, float2, RSET>(sm, ldz, 3 * nt, J.fz.plan, J.fz.tw_f, 0, blockDim.x);
+  // layers [nz, Qz) are zero padding: the first stage takes them as zero unread
+  fft_smem<kFwdDif, float2, RSET>(sm, ldz, 3 * nt, J.fz.plan, J.fz.tw_f, 0, blockDim.x, nz);
 
-  // spectral products at the pair (kz, Qz - kz) of every y position of the tile
+  // spectral products at the pair (kz, Qz - kz): a warp per y position, its
+  // lanes along kz, the kernel values of the next 32 kz on their way meanwhile
   const int half = Qz >> 1;
   const size_t kstride = (size_t)J.kxh * J.kyq * J.kzq;
-  for (int i = threadIdx.x; i < nt * (half + 1); i += blockDim.x) {
-    const int t = i / (half + 1), kz = i - t * (half + 1);
-    const int ky = fft_freq(y0 + t, J.fy.plan);
+  for (int t = warp; t < nt; t += warps) {
+    const int ky = __ldg(J.fy.freq + y0 + t);
     const bool ym = 2 * ky > Qy;
-    const int kys = ym ? Qy - ky : ky;
-    const bool two = kz != 0 && 2 * kz != Qz;
-    const int q0 = fft_pos(kz, J.fz.plan);
-    const int q1 = two ? fft_pos(Qz - kz, J.fz.plan) : q0;
-    const size_t koff = ((size_t)kx * J.kyq + kys) * J.kzq + kz;
-    float nv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sv[3] = {0.f, 0.f, 0.f};
-    if (J.do_H)
-#pragma unroll
-      for (int c = 0; c < 6; ++c) nv[c] = __ldg(J.N3 + c * kstride + koff);
-    if (J.do_C)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) sv[c] = __ldg(J.S3 + c * kstride + koff);
     const float sy = ym ? -1.f : 1.f;
+    const size_t krow = ((size_t)kx * J.kyq + (ym ? Qy - ky : ky)) * J.kzq;
+    float2* line = sm + 3 * t * ldz;
+    for (int kz = lane; kz <= half; kz += 32) {
+      const bool two = kz != 0 && 2 * kz != Qz;
+      const int q0 = __ldg(J.fz.pos + kz);
+      const int q1 = two ? __ldg(J.fz.pos + Qz - kz) : q0;
+      float nv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sv[3] = {0.f, 0.f, 0.f};
+      if (J.do_H)
 #pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      if (side == 1 && !two) break;
-      const int q = side ? q1 : q0;
-      const float sz = side ? -1.f : 1.f;
-      const float2 mx = sm[(t * 3 + 0) * ldz + q], my = sm[(t * 3 + 1) * ldz + q],
-                   mz = sm[(t * 3 + 2) * ldz + q];
-      if (J.do_C) {
-        // phi = i (Sx mx + Sy my + Sz mz); Sy odd in y, Sz odd in z
-        const float ax = sv[0], ay = sy * sv[1], az = sz * sv[2];
-        phi[t * ldz + q] = c_i_times(make_float2(ax * mx.x + ay * my.x + az * mz.x,
-                                                 ax * mx.y + ay * my.y + az * mz.y));
-      }
-      if (J.do_H) {
-        // N real: xy odd in y, xz odd in z, yz odd in both
-        const float nxx = nv[0], nyy = nv[1], nzz = nv[2];
-        const float nxy = sy * nv[3], nxz = sz * nv[4], nyz = sy * sz * nv[5];
-        sm[(t * 3 + 0) * ldz + q] = make_float2(nxx * mx.x + nxy * my.x + nxz * mz.x,
-                                                nxx * mx.y + nxy * my.y + nxz * mz.y);
-        sm[(t * 3 + 1) * ldz + q] = make_float2(nxy * mx.x + nyy * my.x + nyz * mz.x,
-                                                nxy * mx.y + nyy * my.y + nyz * mz.y);
-        sm[(t * 3 + 2) * ldz + q] = make_float2(nxz * mx.x + nyz * my.x + nzz * mz.x,
-                                                nxz * mx.y + nyz * my.y + nzz * mz.y);
+        for (int c = 0; c < 6; ++c) nv[c] = __ldg(J.N3 + c * kstride + krow + kz);
+      if (J.do_C)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sv[c] = __ldg(J.S3 + c * kstride + krow + kz);
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        if (side == 1 && !two) break;
+        const int q = side ? q1 : q0;
+        const float sz = side ? -1.f : 1.f;
+        const float2 mx = line[q], my = line[ldz + q], mz = line[2 * ldz + q];
+        if (J.do_C) {
+          // phi = i (Sx mx + Sy my + Sz mz); Sy odd in y, Sz odd in z
+          const float ax = sv[0], ay = sy * sv[1], az = sz * sv[2];
+          phi[t * ldz + q] = c_i_times(make_float2(ax * mx.x + ay * my.x + az * mz.x,
+                                                   ax * mx.y + ay * my.y + az * mz.y));
+        }
+        if (J.do_H) {
+          // N real: xy odd in y, xz odd in z, yz odd in both
+          const float nxx = nv[0], nyy = nv[1], nzz = nv[2];
+          const float nxy = sy * nv[3], nxz = sz * nv[4], nyz = sy * sz * nv[5];
+          line[q] = make_float2(nxx * mx.x + nxy * my.x + nxz * mz.x, nxx * mx.y + nxy * my.y + nxz * mz.y);
+          line[ldz + q] = make_float2(nxy * mx.x + nyy * my.x + nyz * mz.x, nxy * mx.y + nyy * my.y + nyz * mz.y);
+          line[2 * ldz + q] = make_float2(nxz * mx.x + nyz * my.x + nzz * mz.x, nxz * mx.y + nyz * my.y + nzz * mz.y);
+        }
       }
     }
   }
@@ -162,29 +191,35 @@ __global__ void __launch_bounds__(256, 2) k_zpass3(const Launch<ZJob> Lc) {
   if (J.do_H) fft_smem<kInvDit, float2, RSET>(sm, ldz, 3 * nt, J.fz.plan, J.fz.tw_f, 0, blockDim.x);
   if (J.do_C) fft_smem<kInvDit, float2, RSET>(phi, ldz, nt, J.fz.plan, J.fz.tw_f, 0, blockDim.x);
 
+  // outputs with the y position fastest: runs of the tile's positions
   if (J.do_H) {
-    for (int i = threadIdx.x; i < P3 * nt; i += blockDim.x) {
-      const int q = i / nt, t = i - q * nt;
-      const int c = q / nz, z = q - c * nz;
-      J.outH[((size_t)q * J.kxh + kx) * Qy + y0 + t] = sm[(t * 3 + c) * ldz + z];
+    for (int c = 0; c < 3; ++c) {
+      float2* out = J.outH + ((size_t)c * nz * J.kxh + kx) * Qy + y0;
+      for (int i = threadIdx.x; i < nz << zl; i += blockDim.x) {
+        const int z = i >> zl, t = i & (zt - 1);
+        if (t < nt) out[(size_t)z * J.kxh * Qy + t] = sm[(t * 3 + c) * ldz + z];
+      }
     }
   }
   if (J.do_C) {
     const int r = J.r;
+    float2* out = J.outC + (size_t)kx * Qy + y0;
+    const size_t ostride = (size_t)J.kxh * Qy;
     if (J.fir) {
       const int nch = (r + kZChunk - 1) / kZChunk;
-      for (int i = threadIdx.x; i < nt * nch; i += blockDim.x) {
-        const int t = i / nch;
-        const int k0 = (i - t * nch) * kZChunk;
+      for (int i = threadIdx.x; i < nch << zl; i += blockDim.x) {
+        const int t = i & (zt - 1);
+        const int k0 = (i >> zl) * kZChunk;
+        if (t >= nt) continue;
         const float2* line = phi + t * ldz;
         prefilter_chunk<kZChunk, f2>(
             k0, r, [&](int jj) { return f2(line[tab[jj]]); },
-            [&](int k, f2 v) { J.outC[((size_t)k * J.kxh + kx) * Qy + y0 + t] = make_float2(v.x, v.y); });
+            [&](int k, f2 v) { out[k * ostride + t] = make_float2(v.x, v.y); });
       }
     } else {
-      for (int i = threadIdx.x; i < nt * r; i += blockDim.x) {
-        const int k = i / nt, t = i - k * nt;
-        J.outC[((size_t)k * J.kxh + kx) * Qy + y0 + t] = phi[t * ldz + tab[k + kPrefWarm]];
+      for (int i = threadIdx.x; i < r << zl; i += blockDim.x) {
+        const int k = i >> zl, t = i & (zt - 1);
+        if (t < nt) out[k * ostride + t] = phi[t * ldz + tab[k + kPrefWarm]];
       }
     }
   }
@@ -205,10 +240,9 @@ __global__ void __launch_bounds__(256, 3) k_yinv3(const Launch<YInvJob> Lc) {
   const int Q = FIXP ? FixedPlan<FIXP ? FIXP : 1>::L : J.fy.plan.L;
   const int ldl = Q + 1;
   int* tab = reinterpret_cast<int*>(sm + J.group * ldl);
-  for (int l = 0; l < np; ++l) {
-    const float2* col = J.in + ((size_t)(p0 + l) * J.kxh + kx) * Q;
-    for (int p = threadIdx.x; p < Q; p += blockDim.x) sm[l * ldl + p] = col[p];
-  }
+  const float2* in0 = J.in + ((size_t)p0 * J.kxh + kx) * Q;
+  const size_t pstride = (size_t)J.kxh * Q;
+  load_lines(sm, ldl, np, Q, [&](int l, int p) { return in0[l * pstride + p]; });
   // natural-order input: DIF stages of the inverse leave the rows in DIF
   // order, read back through the position table; DIF-order input: DIT stages
   // leave natural order
@@ -429,8 +463,14 @@ cudaError_t launch_zmix3(const Launch<ZMixJob>& L, cudaStream_t st) {
 
 // ------------------------------------------------------------------ host side
 // about 80 KB of lines per CTA (two CTAs per SM), at least 8 y positions:
-// short z grids get many positions, which spreads the per-CTA set-up
-int zpass_tile(int Qz) { return std::max(8, (80 * 1024) / (4 * (Qz + 1) * (int)sizeof(float2))); }
+// short z grids get many positions, which spreads the per-CTA set-up.  A power
+// of two: whole 64-byte runs and no divisions in the output loops.
+int zpass_tile(int Qz) {
+  const int most = std::max(8, (84 * 1024) / (4 * (Qz + 1) * (int)sizeof(float2)));
+  int t = 8;
+  while (2 * t <= most) t *= 2;
+  return t;
+}
 int zpass_tiles(int Qy, int ztile) { return (Qy + ztile - 1) / ztile; }
 
 // every job's y plan is 1080 = 12 6 15 (fixed plan 2: the 512 x 512 films)
