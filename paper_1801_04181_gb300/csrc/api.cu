@@ -935,7 +935,7 @@ mm_status ensure_plan(mm_ctx* ctx) {
       } else {
         if ((size_t)(S.Qy + 1) * sizeof(float2) + 4096 > 220 * 1024)
           return fail(ctx, MM_ENOTSUP, "y extent too large for one shared-memory line");
-        if (zfft && (size_t)4 * zpass_tile(S.Qz) * (S.Qz + 1) * sizeof(float2) + 8192 > 220 * 1024)
+        if (zfft && (size_t)4 * 8 * (S.Qz + 1) * sizeof(float2) + 8192 > 220 * 1024)
           return fail(ctx, MM_ENOTSUP, "z extent too large for the z pass");
       }
       S.Nq_Ms = 0;  // force a spectra rebuild
@@ -1183,7 +1183,7 @@ mm_status run_source_passes(mm_ctx* ctx, const float* in[2], const int* which, i
       }
       if (S.zfft) {
         FftTables fz;
-        CKS(get_fft(ctx, S.Qz, &fz));
+        CKS(get_fft(ctx, S.Qz, &fz, true));
         ZJob& Z = Lz.job[nzj];
         Z.in = S.Y3; Z.nz = S.nz; Z.kxh = S.kxh; Z.fy = fy; Z.fz = fz; Z.kyq = S.kyq; Z.kzq = S.kzq;
         Z.N3 = S.N3; Z.S3 = S.S3;

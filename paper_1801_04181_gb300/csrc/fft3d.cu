@@ -112,92 +112,117 @@ __global__ void __launch_bounds__(256, 3) k_yfwd3(const Launch<YFwdJob> Lc) {
 }
 
 // ------------------------------------------------------------------ z pass
-__device__ __forceinline__ float2 c_i_times(float2 m) { return make_float2(-m.y, m.x); }
-
-template <unsigned RSET>
-__global__ void __launch_bounds__(256, 2) k_zpass3(const Launch<ZJob> Lc) {
-  extern __shared__ float2 sm[];
+// Two neighbouring y positions are a pair of lines per component (fft2.cuh).
+constexpr int kZThreads = 384;  // two CTAs per SM
+template <typename Fft>
+__global__ void __launch_bounds__(kZThreads, 2) k_zpass3(const Launch<ZJob> Lc) {
+  extern __shared__ float4 sm4[];
   pdl_wait();
   const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
   const ZJob& J = Lc.job[j];
   const int tile = blockIdx.x - Lc.tile_start[j];
-  const int Qy = J.fy.plan.L, Qz = J.fz.plan.L;
+  const int Qy = J.fy.plan.L, Qz = Fft::kL ? Fft::kL : J.fz.plan.L;
   const int zt = J.ztile;
   const int zl = 31 - __clz(zt);  // zt is a power of two
   const int npt = (Qy + zt - 1) >> zl;
   const int kx = tile / npt;
   const int y0 = (tile - kx * npt) << zl;
-  const int nt = min(zt, Qy - y0);
+  const int nt = min(zt, Qy - y0);  // even, as Qy is
+  const int np = nt >> 1;           // pairs of positions
   const int nz = J.nz, P3 = 3 * nz;
   const int ldz = Qz + 1;
-  // lines: t * 3 + c (input, then H in place) for t < nt; phi line t at 3 zt + t
-  float2* phi = sm + 3 * zt * ldz;
-  int* tab = reinterpret_cast<int*>(sm + 4 * zt * ldz);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  // lines: pair * 3 + c (input, then H in place), then the phi line of each pair
+  const int nin = 3 * np;
+  float4* phi = sm4 + nin * ldz;
+  float4* tws = sm4 + 2 * zt * ldz;
+  int* tab = reinterpret_cast<int*>(tws + J.fz.ntw2);
 
-  // the 3 nz values of a y position are one run in memory, nz of each component
+  // the 3 nz values of a y position are one run in memory, nz of each
+  // component; layers [nz, Qz) are zero padding
   const float2* src = J.in + ((size_t)kx * Qy + y0) * P3;
-  load_lines(sm, ldz, 3 * nt, nz, [&](int l, int z) { return src[(size_t)l * nz + z]; });
-  if (J.do_C) build_pref_table(tab, J.r + 2 * kPrefWarm + kZChunk, J.box_lo, J.box_len, J.start, Qz, nullptr);
-  __syncthreads();
-  // layers [nz, Qz) are zero padding: the first stage takes them as zero unread
-  fft_smem<kFwdDif, float2, RSET>(sm, ldz, 3 * nt, J.fz.plan, J.fz.tw_f, 0, blockDim.x, nz);
+  Fft::template in<kFwdDif>(
+      sm4, ldz, nin, J.fz, tws,
+      [&](int l, int z0, int M, auto& v) {
+        const int tp = l / 3, c = l - 3 * tp;
+        const float2* a = src + (size_t)(2 * tp) * P3 + c * nz + z0;
+#pragma unroll
+        for (int k = 0; k < (int)(sizeof(v) / sizeof(v[0])); ++k)
+          v[k] = z0 + k * M < nz ? c2_make(__ldg(a + k * M), __ldg(a + k * M + P3)) : c2_zero();
+      },
+      [&]() {
+        for (int i = threadIdx.x; i < J.fz.ntw2; i += blockDim.x) tws[i] = __ldg(J.fz.tw2 + i);
+        if (J.do_C)
+          build_pref_table(tab, J.r + 2 * kPrefWarm + kZChunk, J.box_lo, J.box_len, J.start, Qz, nullptr);
+      });
 
-  // spectral products at the pair (kz, Qz - kz): a warp per y position, its
-  // lanes along kz, the kernel values of the next 32 kz on their way meanwhile
+  // spectral products at the pair (kz, Qz - kz): lanes along kz, warps along
+  // the position pairs
   const int half = Qz >> 1;
   const size_t kstride = (size_t)J.kxh * J.kyq * J.kzq;
-  for (int t = warp; t < nt; t += warps) {
-    const int ky = __ldg(J.fy.freq + y0 + t);
-    const bool ym = 2 * ky > Qy;
-    const float sy = ym ? -1.f : 1.f;
-    const size_t krow = ((size_t)kx * J.kyq + (ym ? Qy - ky : ky)) * J.kzq;
-    float2* line = sm + 3 * t * ldz;
-    for (int kz = lane; kz <= half; kz += 32) {
-      const bool two = kz != 0 && 2 * kz != Qz;
-      const int q0 = __ldg(J.fz.pos + kz);
-      const int q1 = two ? __ldg(J.fz.pos + Qz - kz) : q0;
-      float nv[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, sv[3] = {0.f, 0.f, 0.f};
-      if (J.do_H)
+  const int lane = threadIdx.x & 31, warps = blockDim.x >> 5;
+  const int runs = (half + 32) >> 5;
+  for (int task = threadIdx.x >> 5; task < np * runs; task += warps) {
+    const int tp = task / runs, kz = ((task - tp * runs) << 5) + lane;
+    if (kz > half) continue;
+    const int kya = __ldg(J.fy.freq + y0 + 2 * tp), kyb = __ldg(J.fy.freq + y0 + 2 * tp + 1);
+    const bool ma = 2 * kya > Qy, mb = 2 * kyb > Qy;
+    const p2 sy = p2_pack(ma ? -1.f : 1.f, mb ? -1.f : 1.f), minus = p2_dup(-1.f);
+    const size_t oa = ((size_t)kx * J.kyq + (ma ? Qy - kya : kya)) * J.kzq + kz;
+    const size_t ob = ((size_t)kx * J.kyq + (mb ? Qy - kyb : kyb)) * J.kzq + kz;
+    p2 nv[6], sv[3];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) nv[c] = __ldg(J.N3 + c * kstride + krow + kz);
-      if (J.do_C)
+    for (int c = 0; c < 6; ++c)
+      nv[c] = J.do_H ? p2_pack(__ldg(J.N3 + c * kstride + oa), __ldg(J.N3 + c * kstride + ob)) : 0ull;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) sv[c] = __ldg(J.S3 + c * kstride + krow + kz);
+    for (int c = 0; c < 3; ++c)
+      sv[c] = J.do_C ? p2_pack(__ldg(J.S3 + c * kstride + oa), __ldg(J.S3 + c * kstride + ob)) : 0ull;
+    // odd in y: S_y, N_xy, N_yz; odd in z (negated at Qz - kz): S_z, N_xz, N_yz
+    sv[1] = p2_mul(sy, sv[1]);
+    nv[3] = p2_mul(sy, nv[3]);
+    nv[5] = p2_mul(sy, nv[5]);
+    const bool two = kz != 0 && 2 * kz != Qz;
+    float4* line = sm4 + 3 * tp * ldz;
 #pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        if (side == 1 && !two) break;
-        const int q = side ? q1 : q0;
-        const float sz = side ? -1.f : 1.f;
-        const float2 mx = line[q], my = line[ldz + q], mz = line[2 * ldz + q];
-        if (J.do_C) {
-          // phi = i (Sx mx + Sy my + Sz mz); Sy odd in y, Sz odd in z
-          const float ax = sv[0], ay = sy * sv[1], az = sz * sv[2];
-          phi[t * ldz + q] = c_i_times(make_float2(ax * mx.x + ay * my.x + az * mz.x,
-                                                   ax * mx.y + ay * my.y + az * mz.y));
-        }
-        if (J.do_H) {
-          // N real: xy odd in y, xz odd in z, yz odd in both
-          const float nxx = nv[0], nyy = nv[1], nzz = nv[2];
-          const float nxy = sy * nv[3], nxz = sz * nv[4], nyz = sy * sz * nv[5];
-          line[q] = make_float2(nxx * mx.x + nxy * my.x + nxz * mz.x, nxx * mx.y + nxy * my.y + nxz * mz.y);
-          line[ldz + q] = make_float2(nxy * mx.x + nyy * my.x + nyz * mz.x, nxy * mx.y + nyy * my.y + nyz * mz.y);
-          line[2 * ldz + q] = make_float2(nxz * mx.x + nyz * my.x + nzz * mz.x, nxz * mx.y + nyz * my.y + nzz * mz.y);
-        }
+    for (int side = 0; side < 2; ++side) {
+      if (side == 1) {
+        if (!two) break;
+        sv[2] = p2_mul(minus, sv[2]);
+        nv[4] = p2_mul(minus, nv[4]);
+        nv[5] = p2_mul(minus, nv[5]);
+      }
+      const int q = __ldg(J.fz.pos + (side ? Qz - kz : kz));
+      const c2 mx = c2_load(line + q), my = c2_load(line + ldz + q), mz = c2_load(line + 2 * ldz + q);
+      if (J.do_C) {  // phi = i (Sx mx + Sy my + Sz mz)
+        const c2 s = c2_axpy(sv[0], mx, c2_axpy(sv[1], my, c2_scale(sv[2], mz)));
+        c2_store(phi + tp * ldz + q, c2_rot4<1>(s));
+      }
+      if (J.do_H) {  // N real
+        c2_store(line + q, c2_axpy(nv[0], mx, c2_axpy(nv[3], my, c2_scale(nv[4], mz))));
+        c2_store(line + ldz + q, c2_axpy(nv[3], mx, c2_axpy(nv[1], my, c2_scale(nv[5], mz))));
+        c2_store(line + 2 * ldz + q, c2_axpy(nv[4], mx, c2_axpy(nv[5], my, c2_scale(nv[2], mz))));
       }
     }
   }
   __syncthreads();
-  if (J.do_H) fft_smem<kInvDit, float2, RSET>(sm, ldz, 3 * nt, J.fz.plan, J.fz.tw_f, 0, blockDim.x);
-  if (J.do_C) fft_smem<kInvDit, float2, RSET>(phi, ldz, nt, J.fz.plan, J.fz.tw_f, 0, blockDim.x);
+  {
+    float4* first = J.do_H ? sm4 : phi;
+    Fft::out(first, ldz, (J.do_H ? nin : 0) + (J.do_C ? np : 0), J.fz, tws, [&](int l, int z0, int M, auto& v) {
+      float4* p = first + (l * ldz + z0);
+#pragma unroll
+      for (int k = 0; k < (int)(sizeof(v) / sizeof(v[0])); ++k) c2_store(p + k * M, v[k]);
+    });
+  }
 
   // outputs with the y position fastest: runs of the tile's positions
+  const int pl = zl - 1;  // log2 of the pairs of a whole tile
   if (J.do_H) {
     for (int c = 0; c < 3; ++c) {
       float2* out = J.outH + ((size_t)c * nz * J.kxh + kx) * Qy + y0;
-      for (int i = threadIdx.x; i < nz << zl; i += blockDim.x) {
-        const int z = i >> zl, t = i & (zt - 1);
-        if (t < nt) out[(size_t)z * J.kxh * Qy + t] = sm[(t * 3 + c) * ldz + z];
+      for (int i = threadIdx.x; i < nz << pl; i += blockDim.x) {
+        const int z = i >> pl, tp = i & ((1 << pl) - 1);
+        if (tp >= np) continue;
+        const float4 v = sm4[(tp * 3 + c) * ldz + z];
+        *reinterpret_cast<float4*>(out + (size_t)z * J.kxh * Qy + 2 * tp) = make_float4(v.x, v.z, v.y, v.w);
       }
     }
   }
@@ -206,20 +231,31 @@ __global__ void __launch_bounds__(256, 2) k_zpass3(const Launch<ZJob> Lc) {
     float2* out = J.outC + (size_t)kx * Qy + y0;
     const size_t ostride = (size_t)J.kxh * Qy;
     if (J.fir) {
+      // one thread per chunk and per real or imaginary part (of both
+      // positions); the two parts swap halves to store whole values
       const int nch = (r + kZChunk - 1) / kZChunk;
-      for (int i = threadIdx.x; i < nch << zl; i += blockDim.x) {
-        const int t = i & (zt - 1);
-        const int k0 = (i >> zl) * kZChunk;
-        if (t >= nt) continue;
-        const float2* line = phi + t * ldz;
-        prefilter_chunk<kZChunk, f2>(
-            k0, r, [&](int jj) { return f2(line[tab[jj]]); },
-            [&](int k, f2 v) { out[k * ostride + t] = make_float2(v.x, v.y); });
+      const int items = nch << zl;
+      for (int base = threadIdx.x & ~31; base < items; base += blockDim.x) {
+        const int idx = min(base + lane, items - 1);  // whole warps swap (items is even)
+        const int part = idx & 1, tp = (idx >> 1) & ((1 << pl) - 1);
+        const int k0 = (idx >> zl) * kZChunk;
+        const bool store = base + lane < items && tp < np;
+        const p2* line = reinterpret_cast<const p2*>(phi + min(tp, np - 1) * ldz) + part;
+        float2* dst = out + 2 * tp + part;
+        prefilter_chunk2<kZChunk>(
+            k0, [&](int jj) { return line[2 * tab[jj]]; },
+            [&](int k, p2 v) {
+              const float2 f = p2_unpack(v);  // (position a, position b) of this part
+              const float other = __shfl_xor_sync(0xffffffffu, part ? f.x : f.y, 1);
+              if (store && k < r) dst[k * ostride] = part ? make_float2(other, f.y) : make_float2(f.x, other);
+            });
       }
     } else {
-      for (int i = threadIdx.x; i < r << zl; i += blockDim.x) {
-        const int k = i >> zl, t = i & (zt - 1);
-        if (t < nt) out[k * ostride + t] = phi[t * ldz + tab[k + kPrefWarm]];
+      for (int i = threadIdx.x; i < r << pl; i += blockDim.x) {
+        const int k = i >> pl, tp = i & ((1 << pl) - 1);
+        if (tp >= np) continue;
+        const float4 v = phi[tp * ldz + tab[k + kPrefWarm]];
+        *reinterpret_cast<float4*>(out + k * ostride + 2 * tp) = make_float4(v.x, v.z, v.y, v.w);
       }
     }
   }
@@ -464,11 +500,15 @@ cudaError_t launch_zmix3(const Launch<ZMixJob>& L, cudaStream_t st) {
 // ------------------------------------------------------------------ host side
 // about 80 KB of lines per CTA (two CTAs per SM), at least 8 y positions:
 // short z grids get many positions, which spreads the per-CTA set-up.  A power
-// of two: whole 64-byte runs and no divisions in the output loops.
+// of two: whole 64-byte runs and no divisions in the output loops.  Four where
+// the longest lines leave no room for the twiddles (at most 2 Qz) and the
+// prefilter table (at most Qz + 37).
 int zpass_tile(int Qz) {
   const int most = std::max(8, (84 * 1024) / (4 * (Qz + 1) * (int)sizeof(float2)));
   int t = 8;
   while (2 * t <= most) t *= 2;
+  const size_t tables = 2 * sizeof(float4) * (size_t)Qz + sizeof(int) * (size_t)(Qz + 2 * kPrefWarm + kZChunk);
+  if (2 * sizeof(float4) * (size_t)t * (Qz + 1) + tables > 227 * 1024) t = 4;
   return t;
 }
 int zpass_tiles(int Qy, int ztile) { return (Qy + ztile - 1) / ztile; }
@@ -497,20 +537,27 @@ cudaError_t launch_yfwd3(const Launch<YFwdJob>& L, cudaStream_t st) {
 
 cudaError_t launch_zpass3(const Launch<ZJob>& L, cudaStream_t st) {
   size_t smem = 0;
+  unsigned rs = 0;
+  bool q160 = true, q288 = true;  // the lengths of 64 and 128 layers, their plans as constants
   for (int i = 0; i < L.njobs; ++i) {
     const ZJob& J = L.job[i];
-    const size_t lines = sizeof(float2) * 4 * J.ztile * (size_t)(J.fz.plan.L + 1);
+    const FftPlanDev& P = J.fz.plan;
+    const size_t lines = sizeof(float4) * (2 * J.ztile * (size_t)(P.L + 1) + J.fz.ntw2);
     const size_t tab = sizeof(int) * (size_t)(J.do_C ? J.r + 2 * kPrefWarm + kZChunk : 0);
     smem = std::max(smem, lines + tab);
+    rs |= plan_radix_set(P);
+    const bool r48 = P.nstages == 3 && P.radix[0] == 4 && P.radix[1] == 8;
+    q160 = q160 && r48 && P.radix[2] == 5;
+    q288 = q288 && r48 && P.radix[2] == 9;
   }
-  unsigned rs = 0;
-  for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set(L.job[i].fz.plan);
-  auto k = (rs & ~kRadixSetA) == 0u ? k_zpass3<kRadixSetA> : k_zpass3<kAllRadices>;
+  auto k = q160   ? k_zpass3<CtPair<4, 8, 5, 1, 1>>
+           : q288 ? k_zpass3<CtPair<4, 8, 9, 1, 1>>
+           : (rs & ~kRadixSetB) == 0u ? k_zpass3<RtPair<kRadixSetB>> : k_zpass3<RtPair<kAllRadices>>;
   cudaError_t e = allow_smem((const void*)k, 227 * 1024);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];
   if (grid == 0) return cudaSuccess;
-  return launch_chained(k, grid, 256, smem, st, L);
+  return launch_chained(k, grid, kZThreads, smem, st, L);
 }
 
 cudaError_t launch_yinv3(const Launch<YInvJob>& L, cudaStream_t st) {
