@@ -200,9 +200,9 @@ def algorithmic_bytes(mm, fp, mixed=False):
     return {0: xf, 1: yp, 2: xi, 3: ga, 4: st}
 
 
-KERNEL_OF_CLASS = {0: ("k_xfwd", ["fft_passes.cu", "fft.cuh", "prefilter.cuh", "umma.cuh", "mm_internal.h"]),
-                   1: ("k_ypass", ["fft_passes.cu", "fft.cuh", "prefilter.cuh", "umma.cuh", "mm_internal.h"]),
-                   2: ("k_xinv", ["fft_passes.cu", "fft.cuh", "prefilter.cuh", "umma.cuh", "mm_internal.h"]),
+KERNEL_OF_CLASS = {0: ("k_xfwd", ["fft_passes.cu", "fft.cuh", "fft2.cuh", "prefilter.cuh", "umma.cuh", "mm_internal.h"]),
+                   1: ("k_ypass", ["fft_passes.cu", "fft.cuh", "fft2.cuh", "prefilter.cuh", "umma.cuh", "mm_internal.h"]),
+                   2: ("k_xinv", ["fft_passes.cu", "fft.cuh", "fft2.cuh", "prefilter.cuh", "umma.cuh", "mm_internal.h"]),
                    3: ("k_gather", ["gather.cu", "dfloat.cuh", "spline_w.cuh", "mm_internal.h"]),
                    4: ("k_stage", ["llg.cu", "mm_internal.h"])}
 

@@ -263,6 +263,8 @@ mm_status mm_assign_lanes(const double* cost, int npairs, int nlanes, int* lane_
  * stages of radices up to 16; among their orderings, the near-fewest modelled
  * shared-memory bank conflicts, then the radix set {4, 9, 15, 16} the pass
  * kernels are also compiled for, then the largest last and first radix.
+ * The passes that run two lines at once (the fused y pass, the z FFT, short x
+ * lines) have orders of their own, of radices up to 12.
  * MM_EINVAL unless L = 2^a 3^b 5^c >= 1; MM_ENOTSUP for plans with too many
  * stages.  Needs no GPU.
  */
@@ -276,7 +278,8 @@ mm_status mm_fft_plan(int L, int radices[8], int* nstages);
  * wavefronts) on the context's own data, `reps` field evaluations each with
  * CUDA events around the passes that use the length, and keeps the fastest
  * for the whole process: contexts created later, and this one, build their
- * tables of that length from it; a length tuned before is reused, not timed
+ * tables of that length from it (the passes on two lines at once only if it
+ * also ran faster than their own order); a length tuned before is reused, not timed
  * again.  Leaves m, the slider and the timing record as they were (the
  * fields of the last evaluation stay in the buffers).  *n_tuned (may be NULL):
  * lengths timed.  Synchronises.  MM_EINVAL for candidates outside 1..16 or

@@ -82,7 +82,8 @@ struct Dir {
   int start[3] = {0, 0, 0}, r[3] = {0, 0, 0}, guard[3] = {0, 0, 0};
   int Tq_box_lo_z = 0, Tq_bz = 0, Tq_start_z = 0, Tq_nout = 0, Tq_prefilter = -1, Tq_Q[2] = {0, 0};
   int Tq_kind = 0;             // 0: S (potential); 1: rows of -N (componentwise field variant)
-  int Tq_stride = 0;           // planes per output (t_stride)
+  int Tq_stride = 0;           // planes per output
+  bool Tq_quads = false;       // quads, or planes (fused_pairs)
   float* Tq = nullptr;
   float2* YC = nullptr;
   float* C = nullptr;
@@ -474,7 +475,8 @@ std::vector<int> plan_pair_radices(int L) {
   long long best_key = -1;
   for (const auto& o : orders) {
     const int m = *std::max_element(o.begin(), o.end());
-    if (m > max_r) continue;
+    // a first radix below four doubles the twiddle table (fused_pairs counts on 4/3 L)
+    if (m > max_r || (o[0] < 4 && *std::max_element(best.begin(), best.end()) >= 4)) continue;
     const long long key = pair_wavefronts(L, o) * 64 + m;
     if (best_key < 0 || key < best_key) {
       best_key = key;
@@ -548,7 +550,7 @@ mm_status get_fft(mm_ctx* ctx, int L, FftTables* out, bool pairs = false) {
   if (r != 1) return fail(ctx, MM_EINVAL, "FFT length is not 2^a 3^b 5^c");
   (void)p2; (void)p3; (void)p5;
   std::vector<int> radix;
-  if (!tuned_plan(L, &radix, pairs)) radix = pairs ? plan_pair_radices(L) : plan_radices(L);
+  if (!tuned_plan(L, &radix, pairs) || (pairs && radix[0] < 4)) radix = pairs ? plan_pair_radices(L) : plan_radices(L);
   if (radix.empty() || (int)radix.size() > kMaxStages)
     return fail(ctx, MM_ENOTSUP, "FFT length has too many factors");
   FftPlanDev P{};
@@ -767,8 +769,10 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   Magnet& S = ctx->mag[s];
   const int n_out = D->r[2];
   const int bz = D->box_len[2];
-  const int tstride = t_stride(S.nz, kind == 0 && !S.thick);  // the fused y pass reads it, or the plane mixing pass
-  if (D->Tq && D->Tq_stride == tstride && D->Tq_box_lo_z == D->box_lo[2] && D->Tq_bz == bz && D->Tq_start_z == D->start[2] &&
+  const bool fused = kind == 0 && !S.thick;  // the fused y pass reads it, else the plane mixing pass
+  const bool quads = !fused || fused_pairs(S.nz, S.Qy);
+  const int tstride = quads ? t_stride(S.nz, fused) : 3 * S.nz;
+  if (D->Tq && D->Tq_stride == tstride && D->Tq_quads == quads && D->Tq_box_lo_z == D->box_lo[2] && D->Tq_bz == bz && D->Tq_start_z == D->start[2] &&
       D->Tq_nout == n_out && D->Tq_prefilter == D->prefilter && D->Tq_Q[0] == S.Qx &&
       D->Tq_Q[1] == S.Qy && D->Tq_kind == kind)
     return MM_OK;
@@ -801,7 +805,7 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   const double scale = S.Ms / ((double)S.Qx * S.Qy);
   if (kind == 0)
     CK(build_T_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], scale, D->box_lo[2], bz, n_out, ctx->W_dev, D->Tq,
-                       tstride, ctx->gen_work, ctx->gen_q, ctx->st));
+                       tstride, quads, ctx->gen_work, ctx->gen_q, ctx->st));
   else  // H = -N M
     CK(build_TN_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], -scale, D->box_lo[2], bz, n_out, ctx->W_dev, D->Tq,
                         ctx->gen_work, ctx->gen_q, ctx->st));
@@ -815,6 +819,7 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   D->Tq_Q[1] = S.Qy;
   D->Tq_kind = kind;
   D->Tq_stride = tstride;
+  D->Tq_quads = quads;
   return MM_OK;
 }
 
@@ -976,7 +981,7 @@ mm_status ensure_plan(mm_ctx* ctx) {
                        std::max(ctx->gen_q_bytes, sizeof(double) * 6 * qsize)));
         const KernelPlan K = kernel_plan(ctx, S);
         CK(build_N_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], -S.Ms / ((double)S.Qx * S.Qy), S.Nq,
-                           ctx->gen_work, ctx->gen_q, ctx->st));
+                           S.thick || fused_pairs(S.nz, S.Qy), ctx->gen_work, ctx->gen_q, ctx->st));
       } else {
         CKS(build_spectra_3d_all(ctx, S, fx, fy));
       }
@@ -1115,7 +1120,7 @@ mm_status run_source_passes(mm_ctx* ctx, const float* in[2], const int* which, i
       YJob& J = L.job[nj];
       J.in = S.X1;
       J.nz = S.nz; J.ny = S.ny; J.kxh = S.kxh; J.kyq = S.kyq;
-      CKS(get_fft(ctx, S.Qy, &J.fy, true));
+      CKS(get_fft(ctx, S.Qy, &J.fy, fused_pairs(S.nz, S.Qy)));
       J.do_H = (what[i] & 1) ? 1 : 0;
       J.Nq = S.Nq;
       J.outH = S.YH;

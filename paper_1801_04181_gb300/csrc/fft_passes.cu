@@ -182,16 +182,13 @@ template <int NZ>
 __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int Q, int nH) {
   // output planes per batch of kernel loads (about 30 values in flight)
   constexpr int OB = 30 / (3 * NZ) > 0 ? 30 / (3 * NZ) : 1;
-  // quads (quad_index): plane p of this column at (p / 2) qs + 2 (p % 2)
-  const size_t qs = (size_t)((J.kxh + 1) >> 1) * J.kyq * 4;
-  auto plane = [&](int p) { return (p >> 1) * qs + 2 * (p & 1); };
-  const int ts = t_stride(NZ, true);
+  const int kstride = J.kxh * J.kyq;  // one stored kernel plane (< 2^31 values in all)
   const int half = Q >> 1;
   for (int kyq = threadIdx.x; kyq <= half; kyq += blockDim.x) {
     // the two frequencies ky = kyq and Qy - kyq share every stored kernel value;
     // the second has the odd-in-y components negated
     const bool two = kyq != 0 && 2 * kyq != Q;
-    const size_t koff = 4 * ((size_t)(kx >> 1) * J.kyq + kyq) + (kx & 1);
+    const int koff = kx * J.kyq + kyq;
     const int p0 = fft_pos(kyq, J.fy.plan);
     const int p1 = two ? fft_pos(Q - kyq, J.fy.plan) : p0;
     float2 mh[2][3][NZ];
@@ -206,7 +203,7 @@ __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int
           for (int jz = 0; jz < NZ; ++jz)
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-              tv[o][jz][c] = ob + o < J.n_out ? __ldg(Tk + plane((ob + o) * ts + jz * 3 + c)) : 0.f;
+              tv[o][jz][c] = ob + o < J.n_out ? __ldg(Tk + (((ob + o) * NZ + jz) * 3 + c) * kstride) : 0.f;
         // c(o) = sum_jz sum_c T_c(o, jz) m_c(jz); T = Ms W (S spectra) / (Qx Qy)
 #pragma unroll
         for (int o = 0; o < OB; ++o) {
@@ -234,7 +231,7 @@ __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int
 #pragma unroll
       for (int comp = 0; comp < 6; ++comp)
 #pragma unroll
-        for (int dz = 0; dz < NZ; ++dz) nv[comp][dz] = __ldg(Nk + plane(dz * 6 + comp));
+        for (int dz = 0; dz < NZ; ++dz) nv[comp][dz] = __ldg(Nk + (dz * 6 + comp) * kstride);
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         const float fy = side ? -1.f : 1.f;
@@ -263,11 +260,13 @@ __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int
   }
 }
 
-// One CTA per kx; every job of a launch has NZ layers.  kYThreads = 288 (nine
+// One column per CTA: four layers, and lines too long for two columns (fused_pairs);
+// kernel spectra by planes.  Every job of a launch has NZ layers.  kYThreads = 288 (nine
 // warps) covers the 271 frequency pairs of a 540-point line in one round of
 // the spectral products.
 constexpr int kYThreads = 288;
-template <int NZ, unsigned RSET>
+// FIX540: every job's y plan is 540 = 4 9 15, run with its lengths as constants.
+template <int NZ, unsigned RSET, bool FIX540>
 __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Launch<YJob> Lc) {
   constexpr int Pin = 3 * NZ;
   extern __shared__ float2 sm[];
@@ -282,6 +281,20 @@ __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Laun
   const int ny = J.ny;
   const float2* col0 = J.in + (size_t)kx * ny;
   const size_t pstride = (size_t)J.kxh * ny;  // one input plane
+
+  // The kernel spectra of this kx column are read only after the forward FFT:
+  // start moving their lines into L2 now (one prefetch per 128-byte line).
+  {
+    const size_t kstride = (size_t)J.kxh * J.kyq;
+    const int lines = (J.kyq + 31) / 32;
+    const int nN = J.do_H ? 6 * NZ : 0;
+    const int nT = J.do_C ? 3 * NZ * J.n_out : 0;
+    for (int i = threadIdx.x; i < (nN + nT) * lines; i += blockDim.x) {
+      const int row = i / lines, ln = i - row * lines;
+      const float* p = row < nN ? J.Nq + (size_t)row * kstride : J.Tq + (size_t)(row - nN) * kstride;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(p + (size_t)kx * J.kyq + 32 * ln));
+    }
+  }
 
   if ((ny & 1) == 0) {
     // one float4 (two complex rows) of every plane per thread and step
@@ -312,10 +325,12 @@ __global__ void __launch_bounds__(kYThreads, NZ <= 2 ? 3 : 2) k_ypass(const Laun
   if (J.do_C)
     build_pref_table(tab, J.r + 2 * kPrefWarm + kYChunk, J.box_lo, J.box_len, J.start, Q, nullptr, J.periodic != 0);
   __syncthreads();
-  fft_smem<kFwdDif, float2, RSET>(sm, Q, Pin, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+  if constexpr (FIX540) fft_smem_fixed<kFwdDif, float2, 4, 9, 15>(sm, Pin, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+  else fft_smem<kFwdDif, float2, RSET>(sm, Q, Pin, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
   ypass_mix<NZ>(J, sm, kx, Q, nH);
   __syncthreads();
-  fft_smem<kInvDit, float2, RSET>(sm, Q, Pout, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+  if constexpr (FIX540) fft_smem_fixed<kInvDit, float2, 4, 9, 15>(sm, Pout, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
+  else fft_smem<kInvDit, float2, RSET>(sm, Q, Pout, J.fy.plan, J.fy.tw_f, 0, blockDim.x);
 
   if (J.do_H) {
     float2* out0 = J.outH + (size_t)kx * ny;
@@ -363,6 +378,7 @@ template <int NZ>
 __device__ __forceinline__ void ypass2_mix(const YJob& J, float4* sm, int kxp, int Q, int cb, int c0, int c1,
                                            bool do_H) {
   constexpr int TS = t_stride(NZ, true);
+  static_assert(NZ <= 3, "four layers run one column per CTA");
   constexpr int OB = NZ == 1 ? 4 : NZ == 2 ? 3 : 1;  // outputs per batch of loads: whole quads
   constexpr int TQ = (OB * TS + 1) / 2;    // their quads
   const unsigned qs = (unsigned)((J.kxh + 1) >> 1) * J.kyq;  // quads of two planes
@@ -961,8 +977,8 @@ static size_t ypass2_smem(const YJob& J, int ch) {
 }
 
 // Coefficient planes at a time: all of them, or the most that let two CTAs
-// share an SM, or the most that fit; 0 if that is none.  Chunks start on whole
-// quads of the kernel spectra: one layer's hold two planes.
+// share an SM, or the most that fit (fused_pairs: two at least).  Chunks start on
+// whole quads of the kernel spectra: one layer's hold two planes.
 static int ypass2_chunk(const YJob& J) {
   const int n_out = J.do_C ? J.n_out : 0;
   for (size_t limit : {kSmemTwo, kSmemMax}) {
@@ -973,71 +989,77 @@ static int ypass2_chunk(const YJob& J) {
   return 0;
 }
 
-template <int NZ>
-static cudaError_t launch_ypass_nz(const Launch<YJob>& L0, size_t smem1, cudaStream_t st) {
+// The jobs of one layer count, two columns per CTA.
+template <int NZ> static cudaError_t launch_ypass_pairs(const Launch<YJob>& L0, cudaStream_t st) {
   Launch<YJob> L = L0;
   unsigned rs = 0;
-  bool pairs = true;
-  int id = -1;
+  int id = -1, tiles = 0;
   size_t smem = 0;
   for (int i = 0; i < L.njobs; ++i) {
     YJob& J = L.job[i];
     rs |= plan_radix_set(J.fy.plan);
     J.ch = ypass2_chunk(J);
+    if (J.ch == 0) return cudaErrorInvalidConfiguration;
     id = id < 0 || id == pair_plan_id(J.fy.plan) ? pair_plan_id(J.fy.plan) : 0;
-    pairs = pairs && J.ch > 0;
     smem = max(smem, ypass2_smem(J, J.ch));
+    L.tile_start[i] = tiles;
+    tiles += (J.kxh + 1) / 2;
   }
-  void (*k)(const Launch<YJob>);
-  int threads = kYThreads;
-  if (pairs) {
-    // the lengths of 64, 128, 256, 512 and 1024 cells (4 cells of margin) with
-    // their plans as constants, 13% faster at 540; else the plan at run time
-    k = id == 1   ? k_ypass2<NZ, CtPair<4, 8, 5>>
-        : id == 2 ? k_ypass2<NZ, CtPair<4, 8, 9>>
-        : id == 3 ? k_ypass2<NZ, CtPair<12, 9, 5>>
-        : id == 4 ? k_ypass2<NZ, CtPair<12, 9, 10>>
-        : id == 5 ? k_ypass2<NZ, CtPair<6, 8, 9, 5>>
-        : (rs & ~kRadixSetB) == 0u ? k_ypass2<NZ, RtPair<kRadixSetB>> : k_ypass2<NZ, RtPair<kAllRadices>>;
-    const int ctas = min(3, max(1, (int)(228 * 1024 / (smem + 1024))));
-    threads = kY2Threads / ctas / 32 * 32;
-    int tiles = 0;
-    for (int i = 0; i < L.njobs; ++i) {
-      L.tile_start[i] = tiles;
-      tiles += (L.job[i].kxh + 1) / 2;
-    }
-    L.tile_start[L.njobs] = tiles;
-  } else {
-    k = (rs & ~kRadixSetA) == 0u ? k_ypass<NZ, kRadixSetA> : k_ypass<NZ, kAllRadices>;
-    smem = smem1;
-  }
+  L.tile_start[L.njobs] = tiles;
+  // the lengths of 64, 128, 256, 512 and 1024 cells (4 cells of margin) with
+  // their plans as constants, 13% faster at 540; else the plan at run time
+  auto k = id == 1   ? k_ypass2<NZ, CtPair<4, 8, 5>>
+           : id == 2 ? k_ypass2<NZ, CtPair<4, 8, 9>>
+           : id == 3 ? k_ypass2<NZ, CtPair<12, 9, 5>>
+           : id == 4 ? k_ypass2<NZ, CtPair<10, 12, 9>>
+           : id == 5 ? k_ypass2<NZ, CtPair<6, 8, 9, 5>>
+           : (rs & ~kRadixSetB) == 0u ? k_ypass2<NZ, RtPair<kRadixSetB>> : k_ypass2<NZ, RtPair<kAllRadices>>;
   cudaError_t e = allow_smem((const void*)k, kSmemMax);
-  if (e != cudaSuccess) return e;
-  const int grid = L.tile_start[L.njobs];
-  if (grid == 0) return cudaSuccess;
-  return launch_chained(k, grid, threads, smem, st, L);
+  if (e != cudaSuccess || tiles == 0) return e;
+  const int ctas = min(3, max(1, (int)(228 * 1024 / (smem + 1024))));
+  return launch_chained(k, tiles, kY2Threads / ctas / 32 * 32, smem, st, L);
 }
 
-// Jobs of different layer counts go to separate launches of the matching kernel.
-cudaError_t launch_ypass(const Launch<YJob>& L, size_t smem, cudaStream_t st) {
-  for (int nz = 1; nz <= kMaxNz; ++nz) {
-    Launch<YJob> S{};
-    int tiles = 0;
-    for (int i = 0; i < L.njobs; ++i) {
-      if (L.job[i].nz != nz) continue;
-      S.job[S.njobs] = L.job[i];
-      S.tile_start[S.njobs] = tiles;
-      tiles += L.tile_start[i + 1] - L.tile_start[i];
-      ++S.njobs;
-    }
-    if (S.njobs == 0) continue;
-    S.tile_start[S.njobs] = tiles;
-    cudaError_t e = nz == 1   ? launch_ypass_nz<1>(S, smem, st)
-                    : nz == 2 ? launch_ypass_nz<2>(S, smem, st)
-                    : nz == 3 ? launch_ypass_nz<3>(S, smem, st)
-                              : launch_ypass_nz<4>(S, smem, st);
-    if (e != cudaSuccess) return e;
+// ... and one column per CTA.
+template <int NZ> static cudaError_t launch_ypass_columns(const Launch<YJob>& L, size_t smem, cudaStream_t st) {
+  unsigned rs = 0;
+  bool fix540 = true;
+  for (int i = 0; i < L.njobs; ++i) {
+    rs |= plan_radix_set(L.job[i].fy.plan);
+    fix540 = fix540 && fixed_plan_id(L.job[i].fy.plan) == 3;
   }
+  auto k = fix540 ? k_ypass<NZ, kRadixSetA, true>
+                  : (rs & ~kRadixSetA) == 0u ? k_ypass<NZ, kRadixSetA, false> : k_ypass<NZ, kAllRadices, false>;
+  cudaError_t e = allow_smem((const void*)k, kSmemMax);
+  if (e != cudaSuccess || L.tile_start[L.njobs] == 0) return e;
+  return launch_chained(k, L.tile_start[L.njobs], kYThreads, smem, st, L);
+}
+
+// Jobs of different layer counts, or of one and two columns per CTA, go to
+// separate launches of the matching kernel.
+cudaError_t launch_ypass(const Launch<YJob>& L, size_t smem, cudaStream_t st) {
+  for (int nz = 1; nz <= kMaxNz; ++nz)
+    for (int pairs = 0; pairs < 2; ++pairs) {
+      Launch<YJob> S{};
+      int tiles = 0;
+      for (int i = 0; i < L.njobs; ++i) {
+        if (L.job[i].nz != nz || fused_pairs(nz, L.job[i].fy.plan.L) != (pairs != 0)) continue;
+        S.job[S.njobs] = L.job[i];
+        S.tile_start[S.njobs] = tiles;
+        tiles += L.job[i].kxh;
+        ++S.njobs;
+      }
+      if (S.njobs == 0) continue;
+      S.tile_start[S.njobs] = tiles;
+      cudaError_t e = pairs ? (nz == 1   ? launch_ypass_pairs<1>(S, st)
+                               : nz == 2 ? launch_ypass_pairs<2>(S, st)
+                                         : launch_ypass_pairs<3>(S, st))
+                      : nz == 1 ? launch_ypass_columns<1>(S, smem, st)
+                      : nz == 2 ? launch_ypass_columns<2>(S, smem, st)
+                      : nz == 3 ? launch_ypass_columns<3>(S, smem, st)
+                                : launch_ypass_columns<4>(S, smem, st);
+      if (e != cudaSuccess) return e;
+    }
   return cudaSuccess;
 }
 

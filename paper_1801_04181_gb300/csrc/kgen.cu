@@ -283,9 +283,9 @@ __global__ void k_extract_quarter(const double2* spec, double* out, int Qx, int 
 }
 
 // T[o][jz][c] = scale * sum_zb W[o][zb] Sq[(zb - jz) - dz_lo][c]  (quarter
-// planes), stored as quads, plane o * tstride + jz * 3 + c
+// planes), plane o * tstride + jz * 3 + c, as quads or by planes
 __global__ void k_mix_T(const double* Sq, const double* W, float* T, int n_out, int nz, int bz,
-                        int dz_first_plane_offset, int kxh, int kyq, int tstride, double scale) {
+                        int dz_first_plane_offset, int kxh, int kyq, int tstride, int quads, double scale) {
   const size_t qsize = (size_t)kxh * kyq;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= qsize) return;
@@ -299,7 +299,8 @@ __global__ void k_mix_T(const double* Sq, const double* W, float* T, int n_out, 
     const int plane = zb - jz + dz_first_plane_offset;
     acc += w * Sq[((size_t)plane * 3 + c) * qsize + i];
   }
-  T[quad_index(o * tstride + jz * 3 + c, (int)(i / kyq), (int)(i % kyq), kxh, kyq)] = (float)(scale * acc);
+  const int p = o * tstride + jz * 3 + c;
+  T[quads ? quad_index(p, (int)(i / kyq), (int)(i % kyq), kxh, kyq) : (size_t)p * qsize + i] = (float)(scale * acc);
 }
 
 // Componentwise field variant: TN[(a n_out + o) nz + jz][b] = scale * sum_zb
@@ -326,11 +327,11 @@ __global__ void k_mix_TN(const double* Nq6, const double* W, float* T, int n_out
       (float)(scale * acc);
 }
 
-// one quarter plane into plane `plane` of a quad array
-__global__ void k_put_quads(const double* in, float* out, int plane, int kxh, int kyq, double scale) {
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < (size_t)kxh * kyq)
-    out[quad_index(plane, (int)(i / kyq), (int)(i % kyq), kxh, kyq)] = (float)(scale * in[i]);
+// one quarter plane into plane `plane` of an array of quads or planes
+__global__ void k_put_plane(const double* in, float* out, int plane, int kxh, int kyq, int quads, double scale) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x, n = (size_t)kxh * kyq;
+  if (i < n)
+    out[quads ? quad_index(plane, (int)(i / kyq), (int)(i % kyq), kxh, kyq) : plane * n + i] = (float)(scale * in[i]);
 }
 
 __global__ void k_scale_to_float(const double* in, float* out, size_t n, double scale) {
@@ -379,7 +380,7 @@ static cudaError_t plane_spectra(int kind, int ncomp, const KernelPlan& K, int d
 }
 
 cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
-                            double b, double c, double scale, float* Nq, double2* work, double* qbuf,
+                            double b, double c, double scale, float* Nq, bool quads, double2* work, double* qbuf,
                             cudaStream_t st) {
   const int kxh = K.Qx / 2 + 1, kyq = K.Qy / 2 + 1;
   const size_t qsize = (size_t)kxh * kyq;
@@ -388,7 +389,8 @@ cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftT
     cudaError_t e = plane_spectra(1, 6, K, dz, a, b, c, fx, fy, work, qbuf, imag6, st);
     if (e != cudaSuccess) return e;
     for (int q = 0; q < 6; ++q)
-      k_put_quads<<<(unsigned)((qsize + 255) / 256), 256, 0, st>>>(qbuf + q * qsize, Nq, dz * 6 + q, kxh, kyq, scale);
+      k_put_plane<<<(unsigned)((qsize + 255) / 256), 256, 0, st>>>(qbuf + q * qsize, Nq, dz * 6 + q, kxh, kyq, quads,
+                                                                        scale);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -397,7 +399,7 @@ cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftT
 
 cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                             double b, double c, double scale, int box_lo_z, int bz, int n_out,
-                            const double* W_dev, float* Tq, int tstride, double2* work, double* Sq,
+                            const double* W_dev, float* Tq, int tstride, bool quads, double2* work, double* Sq,
                             cudaStream_t st) {
   const int kxh = K.Qx / 2 + 1, kyq = K.Qy / 2 + 1;
   const size_t qsize = (size_t)kxh * kyq;
@@ -411,7 +413,7 @@ cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftT
   }
   // plane index of offset dz = (box_lo_z + zb) - jz is (zb - jz) + (nz - 1)
   dim3 g((unsigned)((qsize + 255) / 256), 3, n_out * K.nz);
-  k_mix_T<<<g, 256, 0, st>>>(Sq, W_dev, Tq, n_out, K.nz, bz, K.nz - 1, kxh, kyq, tstride, scale);
+  k_mix_T<<<g, 256, 0, st>>>(Sq, W_dev, Tq, n_out, K.nz, bz, K.nz - 1, kxh, kyq, tstride, quads, scale);
   return cudaGetLastError();
 }
 

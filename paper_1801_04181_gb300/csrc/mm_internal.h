@@ -49,6 +49,16 @@ __host__ __device__ inline size_t quad_index(int plane, int kx, int ky, int kxh,
 __host__ __device__ inline size_t quad_floats(int planes, int kxh, int kyq) {
   return (size_t)((planes + 1) >> 1) * ((kxh + 1) >> 1) * kyq * 4;
 }
+// Whether the fused y pass takes two columns per CTA: up to three layers (four
+// spill its 80 registers: 400 x 200 x 4 181 -> 229 us a call) where the lines of the
+// inputs and two outputs fit a CTA's shared memory beside the tables (twiddles
+// at most 4/3 Qy: pair plans start with a radix of four or more; prefilter
+// indices at most Qy + 37).  Its kernel spectra are quads
+// then; for one column per CTA they are planes [plane][kx][ky], plane numbers alike
+// with 3 nz planes per output of T.
+__host__ __device__ constexpr bool fused_pairs(int nz, int Qy) {
+  return nz <= 3 && (size_t)(3 * nz + 2) * Qy * 16 + 26 * (size_t)Qy + 512 <= 227 * 1024;
+}
 // planes of N: dz * 6 + component; planes of T: o * stride + jz * 3 + c, the
 // stride even (whole quads per output) except for the fused pass on one layer,
 // which takes two outputs at a time
@@ -88,12 +98,12 @@ struct YJob {
   int kyq;                // Qy/2 + 1 stored ky values of the kernel spectra
   // self-demag output
   int do_H;
-  const float* Nq;        // quads, planes dz * 6 + (xx yy zz xy xz yz), dz >= 0
+  const float* Nq;        // quads or planes (fused_pairs), dz * 6 + (xx yy zz xy xz yz), dz >= 0
   float2* outH;           // [3 nz][kxh][ny]
   // potential / coefficient output
   int do_C;
   int n_out;
-  const float* Tq;        // quads, planes o * t_stride(nz, true) + jz * 3 + c
+  const float* Tq;        // o * t_stride(nz, true) + jz * 3 + c (planes: o * 3 nz + ...)
   float2* outC;           // [n_out][kxh][r]
   int box_lo, box_len, start, r, fir;
   int periodic;           // the y box is the whole period: the prefilter wraps
@@ -464,8 +474,8 @@ cudaError_t launch_mech(const MechParams& P, cudaStream_t st);
 cudaError_t eval_points_fp64(int kind, int n, const double* off_dev, double a, double b, double c,
                              double* out_dev, cudaStream_t st);
 cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
-                            double b, double c, double scale, float* Nq, double2* work, double* qbuf,
-                            cudaStream_t st);  // quads (quad_index)
+                            double b, double c, double scale, float* Nq, bool quads, double2* work, double* qbuf,
+                            cudaStream_t st);
 // 3D spectra of S (kind 0, 3 comps) or N (kind 1, 6 comps): out [comp][kxh][kyq][kzq].
 // Scratch: work 2 * ncomp * Qx * Qy double2, q2 ncomp * Qz * kxh * kyq double,
 // qtmp ncomp * kxh * kyq double, zl kxh * kyq * Qz double2.
@@ -486,7 +496,7 @@ cudaError_t build_S_planes(const KernelPlan& K, const FftTables& fx, const FftTa
                            double* qtmp, cudaStream_t st);
 cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                             double b, double c, double scale, int box_lo_z, int bz, int n_out,
-                            const double* W_dev, float* Tq, int tstride, double2* work, double* Sq,
-                            cudaStream_t st);  // quads
+                            const double* W_dev, float* Tq, int tstride, bool quads, double2* work, double* Sq,
+                            cudaStream_t st);
 
 }  // namespace mm
