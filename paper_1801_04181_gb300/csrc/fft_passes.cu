@@ -465,8 +465,8 @@ __device__ __forceinline__ void ypass2_mix(const YJob& J, float4* sm, int kxp, i
 // planes, in place) and `ch` coefficient planes at a time.
 //
 // What bounds it: shared memory and the latency of the kernel spectra between
-// the barriers (stick-slip films: 46% of the shared-memory wavefronts, 37%
-// issue-active, 17% DRAM).  Against the one-column pass, 45 M warp instructions
+// the barriers (stick-slip films: 46% of the shared-memory wavefronts, 40%
+// issue-active, 20% DRAM).  Against the one-column pass, 40 M warp instructions
 // for 64 M and 94 -> 92 us there; one 1024 x 1024 film over another (one CTA
 // per SM in both) 411 -> 322 us, 355 x 145 x 3 over 301 x 127 x 2 37 + 26 -> 26 +
 // 23 us, 64 x 64 x 1 19 -> 13 us.  640 or 512 threads per SM (fewer, with more
