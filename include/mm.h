@@ -270,6 +270,13 @@ mm_status mm_assign_lanes(const double* cost, int npairs, int nlanes, int* lane_
  */
 mm_status mm_fft_plan(int L, int radices[8], int* nstages);
 
+/* The planner's order of the passes that run two lines at once (arguments and
+ * status as for mm_fft_plan): fewest stages of radices up to 12, the first four
+ * or more where it can be, then the fewest modelled bank conflicts.
+ * *compiled (may be NULL): 1 if the fused y pass has a build for this plan, its
+ * lengths constants; 0 if it runs it with the plan as data.  Needs no GPU. */
+mm_status mm_fft_pair_plan(int L, int radices[8], int* nstages, int* compiled);
+
 /*
  * Autotuner of the FFT plans (the batched form's schedule choice; the paper
  * has no counterpart).  For every transform length this context's pass

@@ -12,7 +12,7 @@ import torch
 from . import _native
 from ._native import MMError, mm_options
 
-__all__ = ["MovingMagnets", "MMError", "assign_lanes", "eval_kernel_fp64", "fft_plan", "load_library", "pair_context",
+__all__ = ["MovingMagnets", "MMError", "assign_lanes", "eval_kernel_fp64", "fft_pair_plan", "fft_plan", "load_library", "pair_context",
            "step_batch", "tuned_plan"]
 
 
@@ -363,6 +363,18 @@ def fft_plan(L):
     if s != 0:
         raise MMError(s, "mm_fft_plan")
     return [r[i] for i in range(n.value)]
+
+
+def fft_pair_plan(L):
+    """mm_fft_pair_plan: (radices, compiled) of the passes that run two lines of
+    length L at once; compiled: the fused y pass has a build for this plan."""
+    lib = _native.load()
+    r = (C.c_int * 8)()
+    n, c = C.c_int(), C.c_int()
+    s = lib.mm_fft_pair_plan(int(L), r, C.byref(n), C.byref(c))
+    if s != 0:
+        raise MMError(s, "mm_fft_pair_plan")
+    return [r[i] for i in range(n.value)], bool(c.value)
 
 
 def tuned_plan(L):

@@ -2661,16 +2661,28 @@ mm_status mm_step_batch(mm_ctx* const* ctxs, int npairs, int nsteps, double* t_o
   return MM_OK;
 }
 
-mm_status mm_fft_plan(int L, int radices[8], int* nstages) {
+// A planner's order for length L into radices[8]; its status as mm_fft_plan's.
+static mm_status plan_query(int L, std::vector<int> (*planner)(int), int radices[8], int* nstages) {
   if (L < 1 || !radices || !nstages) return MM_EINVAL;
   int r = L;
   for (int p : {2, 3, 5})
     while (r % p == 0) r /= p;
   if (r != 1) return MM_EINVAL;
-  const std::vector<int> plan = plan_radices(L);
+  const std::vector<int> plan = planner(L);
   if ((int)plan.size() > kMaxStages || plan.size() > 8) return MM_ENOTSUP;
   *nstages = (int)plan.size();
   for (size_t i = 0; i < plan.size(); ++i) radices[i] = plan[i];
+  return MM_OK;
+}
+
+mm_status mm_fft_plan(int L, int radices[8], int* nstages) { return plan_query(L, plan_radices, radices, nstages); }
+
+mm_status mm_fft_pair_plan(int L, int radices[8], int* nstages, int* compiled) {
+  CKS(plan_query(L, plan_pair_radices, radices, nstages));
+  FftPlanDev P{};
+  P.nstages = *nstages;
+  std::copy(radices, radices + *nstages, P.radix);
+  if (compiled) *compiled = ypass_plan_compiled(P) ? 1 : 0;
   return MM_OK;
 }
 

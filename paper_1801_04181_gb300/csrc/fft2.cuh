@@ -393,6 +393,10 @@ template <unsigned RSET> struct RtPair {
 // L + PAD.
 template <int R0, int R1, int R2, int R3 = 1, int PAD = 0> struct CtPair {
   static constexpr int kL = R0 * R1 * R2 * R3, ldl = kL + PAD;
+  static bool is(const FftPlanDev& P) {
+    return P.nstages == (R3 > 1 ? 4 : 3) && P.radix[0] == R0 && P.radix[1] == R1 && P.radix[2] == R2 &&
+           (R3 == 1 || P.radix[3] == R3);
+  }
   template <int MODE, typename Ld, typename Also>
   static __device__ __forceinline__ void in(float4* buf, int, int nlines, const FftTables& T, const float4* tw, Ld ld,
                                             Also also) {
@@ -420,6 +424,28 @@ template <int R0, int R1, int R2, int R3 = 1, int PAD = 0> struct CtPair {
     __syncthreads();
     fft2_last<R0>(CtStage<R0, kL, kL>(), buf, ldl, nlines, tw, st);
     __syncthreads();
+  }
+};
+
+// The plans a pass on pair lines is compiled for.  A build is taken where every
+// job's plan is its own, stage by stage (CtPair::is): a plan and the stages run
+// over its tables cannot differ.  Else the plan at run time.
+template <typename... Plans> struct PairPlans {
+  static bool has(const FftPlanDev& P) { return (Plans::is(P) || ...); }
+  // the kernel Pass::build<Fft>() of a launch, whose jobs hold the tables `t`
+  template <typename Pass, typename JobT>
+  static auto kernel(const Launch<JobT>& L, FftTables JobT::*t) {
+    unsigned rs = 0;
+    for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set((L.job[i].*t).plan);
+    auto k = (rs & ~kRadixSetB) == 0u ? Pass::template build<RtPair<kRadixSetB>>()
+                                      : Pass::template build<RtPair<kAllRadices>>();
+    auto all = [&](bool (*is)(const FftPlanDev&)) {
+      for (int i = 0; i < L.njobs; ++i)
+        if (!is((L.job[i].*t).plan)) return false;
+      return true;
+    };
+    ((void)(all(&Plans::is) ? (void)(k = Pass::template build<Plans>()) : (void)0), ...);
+    return k;
   }
 };
 

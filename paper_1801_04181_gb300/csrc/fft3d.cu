@@ -535,24 +535,22 @@ cudaError_t launch_yfwd3(const Launch<YFwdJob>& L, cudaStream_t st) {
   return launch_chained(k, grid, 256, smem, st, L);
 }
 
+// the lengths of 64 and 128 layers, their plans as constants
+using ZPairPlans = PairPlans<CtPair<4, 8, 5, 1, 1>, CtPair<4, 8, 9, 1, 1>>;
+struct ZPass3 {
+  template <typename Fft> static auto build() { return &k_zpass3<Fft>; }
+};
+
 cudaError_t launch_zpass3(const Launch<ZJob>& L, cudaStream_t st) {
   size_t smem = 0;
-  unsigned rs = 0;
-  bool q160 = true, q288 = true;  // the lengths of 64 and 128 layers, their plans as constants
   for (int i = 0; i < L.njobs; ++i) {
     const ZJob& J = L.job[i];
     const FftPlanDev& P = J.fz.plan;
     const size_t lines = sizeof(float4) * (2 * J.ztile * (size_t)(P.L + 1) + J.fz.ntw2);
     const size_t tab = sizeof(int) * (size_t)(J.do_C ? J.r + 2 * kPrefWarm + kZChunk : 0);
     smem = std::max(smem, lines + tab);
-    rs |= plan_radix_set(P);
-    const bool r48 = P.nstages == 3 && P.radix[0] == 4 && P.radix[1] == 8;
-    q160 = q160 && r48 && P.radix[2] == 5;
-    q288 = q288 && r48 && P.radix[2] == 9;
   }
-  auto k = q160   ? k_zpass3<CtPair<4, 8, 5, 1, 1>>
-           : q288 ? k_zpass3<CtPair<4, 8, 9, 1, 1>>
-           : (rs & ~kRadixSetB) == 0u ? k_zpass3<RtPair<kRadixSetB>> : k_zpass3<RtPair<kAllRadices>>;
+  auto k = ZPairPlans::kernel<ZPass3>(L, &ZJob::fz);
   cudaError_t e = allow_smem((const void*)k, 227 * 1024);
   if (e != cudaSuccess) return e;
   const int grid = L.tile_start[L.njobs];

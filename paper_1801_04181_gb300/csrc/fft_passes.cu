@@ -919,22 +919,17 @@ template <typename JobT> static bool x_pairs(const Launch<JobT>& L, int tab, siz
   return small;
 }
 // the length of 64 cells (4 cells of margin) with its plan as constants
-#define MM_X_PAIR_BUILDS(K)                                                                  \
-  (x_pair160(L) ? K<CtPair<4, 8, 5, 1, kLinePad>>                                            \
-                : (rs & ~kRadixSetB) == 0u ? K<RtPair<kRadixSetB>> : K<RtPair<kAllRadices>>)
-template <typename JobT> static bool x_pair160(const Launch<JobT>& L) {
-  for (int i = 0; i < L.njobs; ++i) {
-    const FftPlanDev& P = L.job[i].fx.plan;
-    if (P.nstages != 3 || P.radix[0] != 4 || P.radix[1] != 8 || P.radix[2] != 5) return false;
-  }
-  return true;
-}
+using XPairPlans = PairPlans<CtPair<4, 8, 5, 1, kLinePad>>;
+struct XFwd2 {
+  template <typename Fft> static auto build() { return &k_xfwd2<Fft>; }
+};
+struct XInv2 {
+  template <typename Fft> static auto build() { return &k_xinv2<Fft>; }
+};
 
 cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st) {
   if (size_t sm2; x_pairs(L, 0, &sm2)) {
-    unsigned rs = 0;
-    for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set(L.job[i].fx.plan);
-    auto k2 = MM_X_PAIR_BUILDS(k_xfwd2);
+    auto k2 = XPairPlans::kernel<XFwd2>(L, &XFwdJob::fx);
     cudaError_t e = allow_smem((const void*)k2, kSmemMax);
     if (e != cudaSuccess || L.tile_start[L.njobs] == 0) return e;
     return launch_chained(k2, L.tile_start[L.njobs], kXPairThreads, sm2, st, L);
@@ -958,16 +953,14 @@ cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st) {
 // fit shared memory.
 constexpr size_t kSmemTwo = (228 * 1024) / 2 - 1024;  // each of two CTAs on an SM
 
-// the pair plans with builds of their own (0: none)
-static int pair_plan_id(const FftPlanDev& P) {
-  static const int plans[][5] = {{3, 4, 8, 5, 0}, {3, 4, 8, 9, 0}, {3, 12, 9, 5, 0}, {3, 12, 9, 10, 0}, {4, 6, 8, 9, 5}};
-  for (int i = 0; i < 5; ++i) {
-    bool same = P.nstages == plans[i][0];
-    for (int s = 0; same && s < P.nstages; ++s) same = P.radix[s] == plans[i][1 + s];
-    if (same) return i + 1;
-  }
-  return 0;
-}
+// the lengths of 64, 128, 256, 512 and 1024 cells (4 cells of margin) with
+// their plans as constants, 13% faster at 540
+using YPairPlans =
+    PairPlans<CtPair<4, 8, 5>, CtPair<4, 8, 9>, CtPair<12, 9, 5>, CtPair<10, 12, 9>, CtPair<6, 8, 9, 5>>;
+template <int NZ> struct YPass2 {
+  template <typename Fft> static auto build() { return &k_ypass2<NZ, Fft>; }
+};
+bool ypass_plan_compiled(const FftPlanDev& P) { return YPairPlans::has(P); }
 
 static size_t ypass2_smem(const YJob& J, int ch) {
   const int n_out = J.do_C ? J.n_out : 0;
@@ -992,28 +985,18 @@ static int ypass2_chunk(const YJob& J) {
 // The jobs of one layer count, two columns per CTA.
 template <int NZ> static cudaError_t launch_ypass_pairs(const Launch<YJob>& L0, cudaStream_t st) {
   Launch<YJob> L = L0;
-  unsigned rs = 0;
-  int id = -1, tiles = 0;
+  int tiles = 0;
   size_t smem = 0;
   for (int i = 0; i < L.njobs; ++i) {
     YJob& J = L.job[i];
-    rs |= plan_radix_set(J.fy.plan);
     J.ch = ypass2_chunk(J);
     if (J.ch == 0) return cudaErrorInvalidConfiguration;
-    id = id < 0 || id == pair_plan_id(J.fy.plan) ? pair_plan_id(J.fy.plan) : 0;
     smem = max(smem, ypass2_smem(J, J.ch));
     L.tile_start[i] = tiles;
     tiles += (J.kxh + 1) / 2;
   }
   L.tile_start[L.njobs] = tiles;
-  // the lengths of 64, 128, 256, 512 and 1024 cells (4 cells of margin) with
-  // their plans as constants, 13% faster at 540; else the plan at run time
-  auto k = id == 1   ? k_ypass2<NZ, CtPair<4, 8, 5>>
-           : id == 2 ? k_ypass2<NZ, CtPair<4, 8, 9>>
-           : id == 3 ? k_ypass2<NZ, CtPair<12, 9, 5>>
-           : id == 4 ? k_ypass2<NZ, CtPair<10, 12, 9>>
-           : id == 5 ? k_ypass2<NZ, CtPair<6, 8, 9, 5>>
-           : (rs & ~kRadixSetB) == 0u ? k_ypass2<NZ, RtPair<kRadixSetB>> : k_ypass2<NZ, RtPair<kAllRadices>>;
+  auto k = YPairPlans::kernel<YPass2<NZ>>(L, &YJob::fy);
   cudaError_t e = allow_smem((const void*)k, kSmemMax);
   if (e != cudaSuccess || tiles == 0) return e;
   const int ctas = min(3, max(1, (int)(228 * 1024 / (smem + 1024))));
@@ -1067,9 +1050,7 @@ cudaError_t launch_xinv(const Launch<XInvJob>& L, int Qmax, cudaStream_t st) {
   int out_max = 0;
   for (int i = 0; i < L.njobs; ++i) out_max = max(out_max, L.job[i].out_len);
   if (size_t sm2; x_pairs(L, out_max + 2 * kPrefWarm + kXChunk, &sm2)) {
-    unsigned rs = 0;
-    for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set(L.job[i].fx.plan);
-    auto k2 = MM_X_PAIR_BUILDS(k_xinv2);
+    auto k2 = XPairPlans::kernel<XInv2>(L, &XInvJob::fx);
     cudaError_t e = allow_smem((const void*)k2, kSmemMax);
     if (e != cudaSuccess || L.tile_start[L.njobs] == 0) return e;
     return launch_chained(k2, L.tile_start[L.njobs], kXPairThreads, sm2, st, L);

@@ -405,6 +405,7 @@ cudaError_t init_fft_constants_passes();
 cudaError_t init_fft_constants_kgen();
 cudaError_t init_fft_constants_3d();
 size_t ypass_table_bytes(int r);
+bool ypass_plan_compiled(const FftPlanDev& P);  // the y pass on column pairs has a build of this plan
 cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st);
 cudaError_t launch_ypass(const Launch<YJob>& L, size_t smem, cudaStream_t st);
 cudaError_t launch_xinv(const Launch<XInvJob>& L, int Qmax, cudaStream_t st);
