@@ -158,7 +158,9 @@ cudaError_t launch_pref_T(float* box, const int bdim[3], cudaStream_t st) {
     int lines = 32;
     while (lines > 1 && sizeof(float) * (size_t)(lines + 1) * L > 200 * 1024) lines /= 2;
     const size_t smem = sizeof(float) * (size_t)(lines + 1) * L;
-    cudaError_t e = cudaFuncSetAttribute(k_pref_T, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // one limit for every launch: a limit of each launch's own would be lowered
+    // under a longer box's launch by another thread's shorter one
+    cudaError_t e = allow_smem((const void*)k_pref_T, 227 * 1024);
     if (e != cudaSuccess) return e;
     k_pref_T<<<(unsigned)((nlines + lines - 1) / lines), 256, smem, st>>>(box, bdim[0], bdim[1], bdim[2], axis, lines);
     e = cudaGetLastError();
