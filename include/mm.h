@@ -280,13 +280,14 @@ mm_status mm_fft_pair_plan(int L, int radices[8], int* nstages, int* compiled);
 /*
  * Autotuner of the FFT plans (the batched form's schedule choice; the paper
  * has no counterpart).  For every transform length this context's pass
- * kernels use, times up to `candidates` radix orderings (the planner's model
- * choice first, then the next orderings by modelled shared-memory
- * wavefronts) on the context's own data, `reps` field evaluations each with
- * CUDA events around the passes that use the length, and keeps the fastest
- * for the whole process: contexts created later, and this one, build their
- * tables of that length from it (the passes on two lines at once only if it
- * also ran faster than their own order); a length tuned before is reused, not timed
+ * kernels use, times up to `candidates` radix orderings (the planner's choice
+ * first, then the next orderings of mm_fft_plan's stages by modelled
+ * shared-memory wavefronts) on the context's own data, `reps` field evaluations
+ * each with CUDA events around the passes that use the length, and keeps the
+ * fastest for the whole process: contexts created later, and this one, build
+ * their tables of that length from it.  The passes on two lines at once are
+ * timed, and keep their order, apart from the passes on single lines; a length
+ * tuned before in passes of the same kind is reused, not timed
  * again.  Leaves m, the slider and the timing record as they were (the
  * fields of the last evaluation stay in the buffers).  *n_tuned (may be NULL):
  * lengths timed.  Synchronises.  MM_EINVAL for candidates outside 1..16 or
@@ -294,7 +295,8 @@ mm_status mm_fft_pair_plan(int L, int radices[8], int* nstages, int* compiled);
  */
 mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned);
 
-/* The radix order mm_autotune chose for length L (first stage first), host
+/* The radix order mm_autotune chose for length L (first stage first), that of the
+ * passes on single lines if they were tuned, else of those on two at once; host
  * only; MM_ESTATE if L has not been tuned in this process. */
 mm_status mm_get_tuned_plan(int L, int radices[8], int* nstages);
 

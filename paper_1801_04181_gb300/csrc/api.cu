@@ -487,43 +487,46 @@ std::vector<int> plan_pair_radices(int L) {
 }
 
 // ------------------------------------------------------------ autotuned plans
-// Process-wide radix order per transform length, chosen by mm_autotune from
-// timed runs of the pass kernels; the planner's model choice otherwise.
-// `pairs`: it also ran faster than the planner's choice for pair lines, so the
-// passes on pair lines take it too.
-struct Tuned {
-  std::vector<int> radix;
-  bool pairs;
-};
+// Process-wide radix orders chosen by mm_autotune, by the passes they were timed
+// in: those on single lines of length L under L, those on pair lines under -L (a
+// radix order that suits the one kind need not suit the other).  A pass whose
+// length was not tuned in passes of its kind takes the planner's choice.
 std::mutex g_tune_mu;
-std::map<int, Tuned> g_tuned;
+std::map<int, std::vector<int>> g_tuned;
 
-bool tuned_plan(int L, std::vector<int>* out, bool pairs = false) {
+bool tuned_plan(int key, std::vector<int>* out) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  auto it = g_tuned.find(L);
-  if (it == g_tuned.end() || (pairs && !it->second.pairs)) return false;
-  if (out) *out = it->second.radix;
+  auto it = g_tuned.find(key);
+  if (it == g_tuned.end()) return false;
+  if (out) *out = it->second;
   return true;
 }
 
-void set_tuned_plan(int L, const std::vector<int>& r, bool pairs) {
+void set_tuned_plan(int key, const std::vector<int>& r) {
   std::lock_guard<std::mutex> lock(g_tune_mu);
-  g_tuned[L] = Tuned{r, pairs};
+  g_tuned[key] = r;
+}
+
+void drop_tuned_plan(int key) {
+  std::lock_guard<std::mutex> lock(g_tune_mu);
+  g_tuned.erase(key);
 }
 
 // The candidates an autotuner times for length L: the model's choice first,
 // then the other orderings of the fewest-stage factorisations by modelled
-// shared-memory wavefronts, at most `k` in all.
-std::vector<std::vector<int>> plan_candidates(int L, int k) {
+// shared-memory wavefronts, at most `k` in all.  `pairs`: for the passes on pair
+// lines, whose own choice comes first and whose first radix is four or more.
+std::vector<std::vector<int>> plan_candidates(int L, int k, bool pairs) {
   std::vector<std::vector<int>> out;
   const std::vector<int> model = plan_radices(L);
   if (model.empty()) return out;
-  out.push_back(model);
+  out.push_back(pairs ? plan_pair_radices(L) : model);
   std::vector<int> cur;
   std::vector<std::vector<int>> orders;
   radix_orders(L, (int)model.size(), cur, orders);
   std::vector<std::pair<long long, std::vector<int>>> w;
-  for (const auto& o : orders) w.push_back({plan_wavefronts(L, o), o});
+  for (const auto& o : orders)
+    if (!pairs || o[0] >= 4) w.push_back({plan_wavefronts(L, o), o});
   std::sort(w.begin(), w.end());
   for (const auto& e : w) {
     if ((int)out.size() >= k) break;
@@ -550,7 +553,7 @@ mm_status get_fft(mm_ctx* ctx, int L, FftTables* out, bool pairs = false) {
   if (r != 1) return fail(ctx, MM_EINVAL, "FFT length is not 2^a 3^b 5^c");
   (void)p2; (void)p3; (void)p5;
   std::vector<int> radix;
-  if (!tuned_plan(L, &radix, pairs) || (pairs && radix[0] < 4)) radix = pairs ? plan_pair_radices(L) : plan_radices(L);
+  if (!tuned_plan(key, &radix)) radix = pairs ? plan_pair_radices(L) : plan_radices(L);
   if (radix.empty() || (int)radix.size() > kMaxStages)
     return fail(ctx, MM_ENOTSUP, "FFT length has too many factors");
   FftPlanDev P{};
@@ -2706,17 +2709,15 @@ mm_status mm_assign_lanes(const double* cost, int npairs, int nlanes, int* lane_
   return MM_OK;
 }
 
-// Drops this context's tables of length L (after its work has drained), so
-// the next launch builds them from the current plan of L.
-static mm_status drop_fft(mm_ctx* ctx, int L) {
+// Drops this context's tables under `key` (after its work has drained), so the
+// next launch builds them from the current plan.
+static mm_status drop_fft(mm_ctx* ctx, int key) {
   CK(cudaStreamSynchronize(ctx->st));
   if (ctx->side) CK(cudaStreamSynchronize(ctx->side));
-  for (int key : {L, -L}) {
-    auto it = ctx->ffts.find(key);
-    if (it == ctx->ffts.end()) continue;
-    cudaFree(it->second.tw_f); cudaFree(it->second.tw_d); cudaFree(it->second.tw2); cudaFree(it->second.pos); cudaFree(it->second.freq);
-    ctx->ffts.erase(it);
-  }
+  auto it = ctx->ffts.find(key);
+  if (it == ctx->ffts.end()) return MM_OK;
+  cudaFree(it->second.tw_f); cudaFree(it->second.tw_d); cudaFree(it->second.tw2); cudaFree(it->second.pos); cudaFree(it->second.freq);
+  ctx->ffts.erase(it);
   return MM_OK;
 }
 
@@ -2725,18 +2726,20 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
     return ctx ? fail(ctx, MM_EINVAL, "mm_autotune") : MM_EINVAL;
   if (n_tuned) *n_tuned = 0;
   CKS(prepare(ctx));
-  // transform lengths of this context and the timing classes of the passes using them
+  // transform lengths of this context (negative: of passes on pair lines) and the
+  // timing classes of the passes using them
   std::map<int, std::set<int>> classes;
   for (const Magnet& S : ctx->mag) {
-    classes[S.Qx].insert(0);
-    classes[S.Qx].insert(2);
+    const int kx = S.Qx <= kXPairMax ? -S.Qx : S.Qx;
+    classes[kx].insert(0);
+    classes[kx].insert(2);
     if (!S.thick) {
-      classes[S.Qy].insert(1);
+      classes[fused_pairs(S.nz, S.Qy) ? -S.Qy : S.Qy].insert(1);
     } else {
       classes[S.Qy].insert(7);
       classes[S.Qy].insert(9);
     }
-    if (S.zfft) classes[S.Qz].insert(8);
+    if (S.zfft) classes[-S.Qz].insert(8);
   }
   // the tuning runs must not disturb the caller's timing record
   const bool timing0 = ctx->timing;
@@ -2759,23 +2762,21 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
     return MM_OK;
   };
   mm_status st = MM_OK;
+  std::set<int> timed;
   for (const auto& kv : classes) {
-    const int L = kv.first;
-    if (L <= 0) continue;
-    if (tuned_plan(L, nullptr)) {  // chosen by an earlier context: use it here too
-      if ((st = drop_fft(ctx, L)) != MM_OK) break;
+    const int key = kv.first, L = std::abs(key);
+    if (L == 0) continue;
+    if (tuned_plan(key, nullptr)) {  // chosen by an earlier context: use it here too
+      if ((st = drop_fft(ctx, key)) != MM_OK) break;
       continue;
     }
-    const auto cands = plan_candidates(L, candidates);
+    const auto cands = plan_candidates(L, candidates, key < 0);
     if (cands.empty()) continue;
-    double best_ms = 0.0, own_ms = 0.0;
+    double best_ms = 0.0;
     size_t best = 0;
-    // the planner's choices first: the passes on pair lines have one of their own
-    if ((st = run()) != MM_OK) break;
-    for (int cls : kv.second) own_ms += ctx->t_ms[cls];
     for (size_t c = 0; c < cands.size() && cands.size() > 1; ++c) {
-      set_tuned_plan(L, cands[c], true);
-      if ((st = drop_fft(ctx, L)) != MM_OK) break;
+      set_tuned_plan(key, cands[c]);
+      if ((st = drop_fft(ctx, key)) != MM_OK) break;
       if ((st = run()) != MM_OK) break;
       double ms = 0.0;
       for (int cls : kv.second) ms += ctx->t_ms[cls];
@@ -2784,11 +2785,15 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
         best = c;
       }
     }
-    if (st != MM_OK) break;
-    set_tuned_plan(L, cands[best], cands.size() > 1 && best_ms < own_ms);
-    if ((st = drop_fft(ctx, L)) != MM_OK) break;
-    if (n_tuned) ++*n_tuned;
+    if (st != MM_OK) {
+      drop_tuned_plan(key);
+      break;
+    }
+    set_tuned_plan(key, cands[best]);
+    if ((st = drop_fft(ctx, key)) != MM_OK) break;
+    timed.insert(L);
   }
+  if (n_tuned) *n_tuned = (int)timed.size();
   drain_timing(ctx);
   std::copy(t_ms0, t_ms0 + kTimingClasses, ctx->t_ms);
   std::copy(t_n0, t_n0 + kTimingClasses, ctx->t_n);
@@ -2799,7 +2804,7 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
 mm_status mm_get_tuned_plan(int L, int radices[8], int* nstages) {
   if (!radices || !nstages) return MM_EINVAL;
   std::vector<int> r;
-  if (!tuned_plan(L, &r)) return MM_ESTATE;
+  if (L < 1 || (!tuned_plan(L, &r) && !tuned_plan(-L, &r))) return MM_ESTATE;
   *nstages = (int)std::min<size_t>(8, r.size());
   for (int i = 0; i < *nstages; ++i) radices[i] = r[i];
   return MM_OK;

@@ -27,3 +27,16 @@ def test_fields_after_tuning_match_oracle(n):
     assert rel_l2(mm.compute_stray_field(0).double().cpu().numpy(), ref["H"]) < TOL
     assert rel_l2(mm.compute_demag(0).double().cpu().numpy(), OF.demag_conv(fp.mat_base.Ms * m0, fp.cell)) < TOL
     mm.close()
+
+
+def test_each_kind_of_pass_keeps_what_was_timed_in_it():
+    """The same lengths in passes on pairs of lines (a film of one layer) and, in y, on
+    single lines (one of six): what the first run kept for y says nothing about the second."""
+    kept = []
+    for n, fresh in (((21, 128, 1), 2), ((21, 128, 6), 1), ((21, 128, 1), 0), ((21, 128, 6), 0)):
+        fp, m0, m1 = workloads.film_pair_plain(n, 2, 4)
+        mm = gpu_pair(fp, m0, m1, mech=False)
+        kept.append(mm.plan_info(0)["fft"])
+        assert mm.autotune(candidates=2, reps=1) == fresh
+        mm.close()
+    assert len(set(kept)) == 1 and kept[0][0] != kept[0][1]
