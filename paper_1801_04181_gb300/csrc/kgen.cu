@@ -361,10 +361,12 @@ static cudaError_t plane_spectra(int kind, int ncomp, const KernelPlan& K, int d
   k_gen_plane<<<g, 128, 0, st>>>(A, kind, Qx, Qy, K.Wx, K.Wy, dz, a, b, c, K.px, K.py, K.R);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  // one limit for every launch: contexts are built from several threads at once
+  e = allow_smem((const void*)k_fft_lines_d, 227 * 1024);
+  if (e != cudaSuccess) return e;
   const int kxh = Qx / 2 + 1, kyq = Qy / 2 + 1;
   for (int q = 0; q < ncomp; ++q) {
     size_t smem = sizeof(double2) * Qx;
-    cudaFuncSetAttribute(k_fft_lines_d, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(sizeof(double2) * (Qx > Qy ? Qx : Qy)));
     k_fft_lines_d<<<Qy, 256, smem, st>>>(A + q * plane, Qy, fx);
     dim3 tg((Qx + 31) / 32, (Qy + 31) / 32);
     k_transpose_d<<<tg, dim3(32, 8), 0, st>>>(A + q * plane, B + q * plane, Qy, Qx);
@@ -512,8 +514,6 @@ cudaError_t build_spectra_3d(int kind, const KernelPlan3& K, const FftTables& fx
       if (e != cudaSuccess) return e;
     }
   }
-  cudaFuncSetAttribute(k_fft_lines_d, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       (int)(sizeof(double2) * std::max(K.Qz, std::max(K.Qx, K.Qy))));
   for (int q = 0; q < ncomp; ++q) {
     dim3 tg((unsigned)((qsize + 31) / 32), (K.Qz + 31) / 32);
     k_zlines<<<tg, dim3(32, 8), 0, st>>>(q2 + (size_t)q * K.Qz * qsize, zl, K.Qz, qsize, imag2d[q]);

@@ -56,3 +56,20 @@ def test_gradients_of_short_and_long_boxes_side_by_side():
     _run([lambda i=i: loop(mms[i], alone[i], streams[i]) for i in range(len(sizes))])
     for mm in mms:
         mm.close()
+
+
+def test_contexts_of_short_and_long_lines_built_side_by_side():
+    """The spectra's set-up transforms whole lines in shared memory: 1 KB for the
+    short films, beyond 48 KB for the long one."""
+
+    def build(n, times):
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            for _ in range(times):
+                mm = _pair(n, stream)
+                H = mm.compute_demag(0)
+                stream.synchronize()
+                assert torch.isfinite(H).all()
+                mm.close()
+
+    _run([lambda: build((1700, 4, 1), 12)] + [lambda: build((6, 5, 1), 60)] * 2)
