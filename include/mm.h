@@ -263,8 +263,8 @@ mm_status mm_assign_lanes(const double* cost, int npairs, int nlanes, int* lane_
  * stages of radices up to 16; among their orderings, the near-fewest modelled
  * shared-memory bank conflicts, then the radix set {4, 9, 15, 16} the pass
  * kernels are also compiled for, then the largest last and first radix.
- * The passes that run two lines at once (the fused y pass, the z FFT, short x
- * lines) have orders of their own, of radices up to 12.
+ * The passes that run two lines at once (the fused y pass, the z FFT) have
+ * orders of their own, of radices up to 12.
  * MM_EINVAL unless L = 2^a 3^b 5^c >= 1; MM_ENOTSUP for plans with too many
  * stages.  Needs no GPU.
  */

@@ -638,9 +638,6 @@ mm_status get_fft(mm_ctx* ctx, int L, FftTables* out, bool pairs = false) {
   return MM_OK;
 }
 
-// the tables of the x passes
-mm_status get_x_fft(mm_ctx* ctx, int L, FftTables* out) { return get_fft(ctx, L, out, L <= kXPairMax); }
-
 double u_cells(const mm_ctx* ctx, int a, double x) {
   return (ctx->u_base[a] + x * ctx->e[a]) / ctx->mag[0].d[a];
 }
@@ -1044,7 +1041,7 @@ Launch<XFwdJob> xfwd_launch(mm_ctx* ctx, const float* in[2], const int* which, i
     J.m = in[which[i]];
     J.out = S.X1;
     J.nx = S.nx; J.ny = S.ny; J.nz = S.nz; J.kxh = S.kxh;
-    get_x_fft(ctx, S.Qx, &J.fx);
+    get_fft(ctx, S.Qx, &J.fx);
     L.tile_start[i] = tiles;
     tiles += (3 * S.nz * S.ny + kRowsPerCta - 1) / kRowsPerCta;
     *Qmax = std::max(*Qmax, S.Qx);
@@ -1306,7 +1303,7 @@ mm_status run_source_passes(mm_ctx* ctx, const float* in[2], const int* which, i
     for (int i = 0; i < n; ++i) {
       Magnet& S = ctx->mag[which[i]];
       FftTables fx;
-      CKS(get_x_fft(ctx, S.Qx, &fx));
+      CKS(get_fft(ctx, S.Qx, &fx));
       if (what[i] & 1) {
         XInvJob& J = L.job[nj];
         J.in = S.YH;
@@ -2092,7 +2089,7 @@ mm_status mm_backward_energy(mm_ctx* ctx, int src, double dE_du[3], float* dE_dm
     CK(cudaMemsetAsync(S.adj_grid, 0, sizeof(float) * (size_t)nzg * S.Qy * S.Qx, st));
     CK(launch_place(S.adj_box, bd, D.box_lo, S.adj_grid, S.Qx, S.Qy, st));
     FftTables fx, fy;
-    CKS(get_x_fft(ctx, S.Qx, &fx));
+    CKS(get_fft(ctx, S.Qx, &fx));
     CKS(get_fft(ctx, S.Qy, &fy));
     {
       Launch<XFwdJob> L{};
@@ -2373,7 +2370,7 @@ mm_status mm_compute_stray_field_componentwise(mm_ctx* ctx, int src, float* H_de
     L.njobs = 1;
     XInvJob& J = L.job[0];
     J.in = D.YC; J.out = D.C; J.planes = PC; J.rows_per_plane = D.r[1]; J.kxh = S.kxh;
-    CKS(get_x_fft(ctx, S.Qx, &J.fx));
+    CKS(get_fft(ctx, S.Qx, &J.fx));
     J.box_lo = D.box_lo[0]; J.box_len = D.box_len[0]; J.start = D.start[0]; J.out_len = D.r[0]; J.fir = 1;
     L.tile_start[1] = (PC * D.r[1] + kRowsPerCta - 1) / kRowsPerCta;
     Timer t(ctx, 2);
@@ -2730,9 +2727,8 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
   // timing classes of the passes using them
   std::map<int, std::set<int>> classes;
   for (const Magnet& S : ctx->mag) {
-    const int kx = S.Qx <= kXPairMax ? -S.Qx : S.Qx;
-    classes[kx].insert(0);
-    classes[kx].insert(2);
+    classes[S.Qx].insert(0);
+    classes[S.Qx].insert(2);
     if (!S.thick) {
       classes[fused_pairs(S.nz, S.Qy) ? -S.Qy : S.Qy].insert(1);
     } else {

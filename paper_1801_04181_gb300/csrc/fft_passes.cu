@@ -704,191 +704,6 @@ __global__ void __launch_bounds__(kXInvThreads, 3) k_xinv(const Launch<XInvJob> 
   }
 }
 
-// ------------------------------------------------------------------ x passes of short lines
-// Lines of at most kXPairMax points on pairs (fft2.cuh): four rows r0 .. r0 + 3 as
-// (r0 + i r1, r2 + i r3), two pairs per CTA.  Short transforms wait on latency,
-// not on arithmetic: these read their first stage straight from memory and keep
-// the later stages' twiddles in shared memory.  64 x 64 x 1 (160 points): forward
-// 7.5 -> 4.8 us, inverse 8.0 -> 5.7 us; 256-point periodic films 22 -> 20 and 35 ->
-// 32 us.  From 300 points on their smaller radices cost more than that gains (300:
-// 38 -> 45 and 48 -> 60 us; 2160: 21 -> 27 and 51 -> 60 us).
-constexpr int kXPairThreads = 256;
-
-template <typename Fft>
-__global__ void __launch_bounds__(kXPairThreads, 3) k_xfwd2(const Launch<XFwdJob> Lc) {
-  extern __shared__ float4 sm4[];
-  pdl_wait();
-  const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
-  const XFwdJob& J = Lc.job[j];
-  const int Q = Fft::kL ? Fft::kL : J.fx.plan.L;
-  const int ldl = Q + kLinePad;
-  const int r0 = (blockIdx.x - Lc.tile_start[j]) * kRowsPerCta;
-  const int nrows = min(kRowsPerCta, 3 * J.nz * J.ny - r0);
-  const int npl = (nrows + 3) >> 2;
-  const int nx = J.nx;
-  const float* row0 = J.m + (size_t)r0 * nx;
-  float4* tws = sm4 + 2 * ldl;
-  // entries [nx, Q) are zero padding, rows past the last of the array too
-  Fft::template in<kFwdDif>(
-      sm4, ldl, npl, J.fx, tws,
-      [&](int pl, int x0, int M, auto& v) {
-        const float* src = row0 + (size_t)(4 * pl) * nx + x0;
-        const int have = nrows - 4 * pl;
-#pragma unroll
-        for (int k = 0; k < (int)(sizeof(v) / sizeof(v[0])); ++k) {
-          const bool in = x0 + k * M < nx;
-          const float a = in ? __ldg(src + k * M) : 0.f, b = in && have > 1 ? __ldg(src + nx + k * M) : 0.f;
-          const float c = in && have > 2 ? __ldg(src + 2 * nx + k * M) : 0.f;
-          const float d = in && have > 3 ? __ldg(src + 3 * nx + k * M) : 0.f;
-          v[k] = c2{p2_pack(a, c), p2_pack(b, d)};
-        }
-      },
-      [&]() {
-        for (int i = threadIdx.x; i < J.fx.ntw2; i += blockDim.x) tws[i] = __ldg(J.fx.tw2 + i);
-      });
-
-  // Z = A + iB:  A_k = (Z_k + conj Z_{Q-k}) / 2,  B_k = (Z_k - conj Z_{Q-k}) / (2i)
-  // thread -> (kx, pair), the pair fastest: a warp writes runs of all the tile's rows
-  const int ny = J.ny, kxh = J.kxh;
-  const p2 h = p2_dup(0.5f), nh = p2_dup(-0.5f);
-  const bool even = (ny & 1) == 0;  // both rows of a line in one plane, 16-byte aligned
-  const int kch = (ny + (int)(kKChunk / 2) - 1) / (int)(kKChunk / 2);
-  for (int i = threadIdx.x; i < kxh * npl; i += blockDim.x) {
-    const int kx = npl == 2 ? i >> 1 : i, pl = npl == 2 ? i & 1 : 0;
-    const float4* line = sm4 + pl * ldl;
-    const c2 zk = c2_load(line + __ldg(J.fx.pos + kx)), zm = c2_load(line + __ldg(J.fx.pos + (kx == 0 ? 0 : Q - kx)));
-    const c2 A = c2{p2_mul(h, p2_add(zk.re, zm.re)), p2_mul(h, p2_sub(zk.im, zm.im))};
-    const c2 B = c2{p2_mul(h, p2_add(zk.im, zm.im)), p2_mul(nh, p2_sub(zk.re, zm.re))};
-    const float2 v[4] = {c2_a(A), c2_a(B), c2_b(A), c2_b(B)};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      if (4 * pl + q >= nrows) break;
-      const int r = r0 + 4 * pl + q, p = r / ny, y = r - p * ny;
-      if (J.pk) {  // reduced precision: straight into the forward DFT's split operand
-        store_split(J.pk, kch, p * kxh + kx, y, v[q]);
-      } else if (!even) {
-        J.out[((size_t)p * kxh + kx) * ny + y] = v[q];
-      } else if ((q & 1) == 0) {  // ny and nrows are even: rows q and q + 1
-        *reinterpret_cast<float4*>(J.out + ((size_t)p * kxh + kx) * ny + y) =
-            make_float4(v[q].x, v[q].y, v[q + 1].x, v[q + 1].y);
-      }
-    }
-  }
-}
-
-// The spectra of a tile's rows staged as the natural-order lines Z = A + iB,
-// transformed in place to digit-reversed order, and read through the plan's
-// positions: demag rows x < nx, or the coefficient rows with the x prefilter.
-template <typename Fft>
-__global__ void __launch_bounds__(kXPairThreads, 3) k_xinv2(const Launch<XInvJob> Lc) {
-  extern __shared__ float4 sm4[];
-  const int j = find_job(Lc.tile_start, Lc.njobs, blockIdx.x);
-  const XInvJob& J = Lc.job[j];
-  const int Q = Fft::kL ? Fft::kL : J.fx.plan.L;
-  const int ldl = Q + kLinePad;
-  const int rpp = J.rows_per_plane, kxh = J.kxh, rows = J.planes * rpp;
-  const int r0 = (blockIdx.x - Lc.tile_start[j]) * kRowsPerCta;
-  const int nrows = min(kRowsPerCta, rows - r0);
-  const int npl = (nrows + 3) >> 2;
-  float4* tws = sm4 + 2 * ldl;
-  int* tab = reinterpret_cast<int*>(tws + J.fx.ntw2);
-  for (int i = threadIdx.x; i < J.fx.ntw2; i += blockDim.x) tws[i] = __ldg(J.fx.tw2 + i);
-  build_pref_table(tab, J.out_len + 2 * kPrefWarm + kXChunk, J.box_lo, J.box_len, J.start, Q, J.fx.pos,
-                   J.periodic != 0);
-  pdl_wait();
-  {
-    // thread -> (kx, pair), the pair fastest: a warp reads runs of all the tile's rows
-    constexpr int kBatchX = 4;
-    const int pl = npl == 2 ? threadIdx.x & 1 : 0;
-    const int have = nrows - 4 * pl;
-    const float2* src[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int r = min(r0 + 4 * pl + q, rows - 1), p = r / rpp;
-      src[q] = J.in + (size_t)p * kxh * rpp + (r - p * rpp);
-    }
-    const bool even = (rpp & 1) == 0;  // both rows of a line in one plane, 16-byte aligned
-    float4* line = sm4 + pl * ldl;
-    const int step = npl == 2 ? blockDim.x >> 1 : blockDim.x;
-    for (int kx0 = npl == 2 ? threadIdx.x >> 1 : threadIdx.x; kx0 < kxh; kx0 += kBatchX * step) {
-      float4 u[kBatchX], w[kBatchX];  // (A, B) of line a, of line b
-#pragma unroll
-      for (int b = 0; b < kBatchX; ++b) {
-        const int kx = kx0 + b * step;
-        u[b] = w[b] = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (kx >= kxh) continue;
-        const size_t o = (size_t)kx * rpp;
-        if (even) {
-          u[b] = *reinterpret_cast<const float4*>(src[0] + o);
-          if (have > 2) w[b] = *reinterpret_cast<const float4*>(src[2] + o);
-        } else {
-          const float2 a0 = src[0][o];
-          u[b].x = a0.x; u[b].y = a0.y;
-          if (have > 1) { const float2 t = src[1][o]; u[b].z = t.x; u[b].w = t.y; }
-          if (have > 2) { const float2 t = src[2][o]; w[b].x = t.x; w[b].y = t.y; }
-          if (have > 3) { const float2 t = src[3][o]; w[b].z = t.x; w[b].w = t.y; }
-        }
-      }
-#pragma unroll
-      for (int b = 0; b < kBatchX; ++b) {
-        const int kx = kx0 + b * step;
-        if (kx >= kxh) continue;
-        // Z_k = A_k + i B_k, Z_{Q-k} = conj A_k + i conj B_k
-        const c2 A = c2{p2_pack(u[b].x, w[b].x), p2_pack(u[b].y, w[b].y)};
-        const c2 B = c2{p2_pack(u[b].z, w[b].z), p2_pack(u[b].w, w[b].w)};
-        c2_store(line + kx, c2_add_i<1>(A, B));
-        if (kx > 0 && 2 * kx != Q) c2_store(line + Q - kx, c2{p2_add(A.re, B.im), p2_sub(B.re, A.im)});
-      }
-    }
-  }
-  __syncthreads();
-  Fft::template in<kInvDif>(
-      sm4, ldl, npl, J.fx, tws,
-      [&](int pl, int n0, int M, auto& v) {
-        const float4* p = sm4 + (pl * ldl + n0);
-#pragma unroll
-        for (int k = 0; k < (int)(sizeof(v) / sizeof(v[0])); ++k) v[k] = c2_load(p + k * M);
-      },
-      [&]() {});
-
-  const int r = J.out_len;
-  float* out0 = J.out + (size_t)r0 * r;
-  if (J.fir) {
-    // one thread per chunk and per real or imaginary part of a pair: rows
-    // 4 pl + part and 4 pl + part + 2
-    const int nch = (r + kXChunk - 1) / kXChunk;
-    for (int idx = threadIdx.x; idx < 2 * npl * nch; idx += blockDim.x) {
-      const int lp = idx / nch, pl = lp >> 1, part = lp & 1;
-      const int k0 = (idx - lp * nch) * kXChunk;
-      const p2* line = reinterpret_cast<const p2*>(sm4 + pl * ldl) + part;
-      const int ra = 4 * pl + part;
-      float* dst = out0 + (size_t)ra * r;
-      const bool one = ra < nrows, other = ra + 2 < nrows;
-      prefilter_chunk2<kXChunk>(
-          k0, [&](int jj) { return line[2 * tab[jj]]; },
-          [&](int k, p2 v) {
-            if (k >= r) return;
-            const float2 f = p2_unpack(v);
-            if (one) dst[k] = f.x;
-            if (other) dst[k + 2 * r] = f.y;
-          });
-    }
-  } else {
-    for (int k = threadIdx.x; k < r; k += blockDim.x) {
-      const int t = tab[k + kPrefWarm];
-      for (int pl = 0; pl < npl; ++pl) {
-        const float4 v = sm4[pl * ldl + t];  // (row 0, row 2, row 1, row 3)
-        float* dst = out0 + (size_t)(4 * pl) * r + k;
-        const int have = nrows - 4 * pl;
-        dst[0] = v.x;
-        if (have > 1) dst[r] = v.z;
-        if (have > 2) dst[2 * r] = v.y;
-        if (have > 3) dst[3 * r] = v.w;
-      }
-    }
-  }
-}
-
 // ------------------------------------------------------------------ host side
 size_t ypass_table_bytes(int r) { return sizeof(int) * (size_t)(r + 2 * kPrefWarm + kYChunk); }
 
@@ -907,33 +722,7 @@ template <typename JobT> static int x_fixed_plan(const Launch<JobT>& L) {
 
 constexpr size_t kSmemMax = 227 * 1024;              // per CTA
 
-// every line of a launch short enough for the pair builds; their shared memory
-template <typename JobT> static bool x_pairs(const Launch<JobT>& L, int tab, size_t* smem) {
-  *smem = 0;
-  bool small = L.njobs > 0;
-  for (int i = 0; i < L.njobs; ++i) {
-    const FftTables& T = L.job[i].fx;
-    small = small && T.plan.L <= kXPairMax;
-    *smem = max(*smem, sizeof(float4) * (2 * (size_t)(T.plan.L + kLinePad) + T.ntw2) + sizeof(int) * (size_t)tab);
-  }
-  return small;
-}
-// the length of 64 cells (4 cells of margin) with its plan as constants
-using XPairPlans = PairPlans<CtPair<4, 8, 5, 1, kLinePad>>;
-struct XFwd2 {
-  template <typename Fft> static auto build() { return &k_xfwd2<Fft>; }
-};
-struct XInv2 {
-  template <typename Fft> static auto build() { return &k_xinv2<Fft>; }
-};
-
 cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st) {
-  if (size_t sm2; x_pairs(L, 0, &sm2)) {
-    auto k2 = XPairPlans::kernel<XFwd2>(L, &XFwdJob::fx);
-    cudaError_t e = allow_smem((const void*)k2, kSmemMax);
-    if (e != cudaSuccess || L.tile_start[L.njobs] == 0) return e;
-    return launch_chained(k2, L.tile_start[L.njobs], kXPairThreads, sm2, st, L);
-  }
   const size_t smem =
       (size_t)kLines * (Qmax + kLinePad) * sizeof(float2) + sizeof(ushort2) * (size_t)(Qmax / 2 + 1);
   unsigned rs = 0;
@@ -1049,12 +838,6 @@ cudaError_t launch_ypass(const Launch<YJob>& L, size_t smem, cudaStream_t st) {
 cudaError_t launch_xinv(const Launch<XInvJob>& L, int Qmax, cudaStream_t st) {
   int out_max = 0;
   for (int i = 0; i < L.njobs; ++i) out_max = max(out_max, L.job[i].out_len);
-  if (size_t sm2; x_pairs(L, out_max + 2 * kPrefWarm + kXChunk, &sm2)) {
-    auto k2 = XPairPlans::kernel<XInv2>(L, &XInvJob::fx);
-    cudaError_t e = allow_smem((const void*)k2, kSmemMax);
-    if (e != cudaSuccess || L.tile_start[L.njobs] == 0) return e;
-    return launch_chained(k2, L.tile_start[L.njobs], kXPairThreads, sm2, st, L);
-  }
   const size_t smem = xinv_smem(Qmax, out_max);
   unsigned rs = 0;
   for (int i = 0; i < L.njobs; ++i) rs |= plan_radix_set(L.job[i].fx.plan);

@@ -10,7 +10,6 @@ constexpr int kMaxJobs = 4;        // jobs per launch (two magnets / two directi
 constexpr int kFirHalf = 14;       // B-spline prefilter FIR half-width, |z1|^15 ~ 2.6e-9
 constexpr int kMaxNz = 4;          // thin-film path: z handled by direct plane mixing
 constexpr int kMaxOut = kMaxNz + 5; // coefficient planes: nz + 3 + 2 guard
-constexpr int kXPairMax = 256;     // the longest x lines that run on pairs (fft2.cuh)
 constexpr int kRowsPerCta = 8;     // real rows per CTA in the x passes (4 complex lines)
 
 // FFT radix sets: one bit per radix the shared-memory FFT implements
