@@ -82,15 +82,16 @@ struct Dir {
   int start[3] = {0, 0, 0}, r[3] = {0, 0, 0}, guard[3] = {0, 0, 0};
   int Tq_box_lo_z = 0, Tq_bz = 0, Tq_start_z = 0, Tq_nout = 0, Tq_prefilter = -1, Tq_Q[2] = {0, 0};
   int Tq_kind = 0;             // 0: S (potential); 1: rows of -N (componentwise field variant)
-  int Tq_stride = 0;           // planes per output
-  bool Tq_quads = false;       // quads, or planes (fused_pairs)
-  float* Tq = nullptr;
+  int Tq_stride = 0;           // planes per output of the quads
+  int Tq_forms = 0;            // the forms held: bit 1 planes, bit 2 quads
+  float* Tq = nullptr;         // planes
+  float* Tqq = nullptr;        // quads
   float2* YC = nullptr;
   float* C = nullptr;
   float2* partial = nullptr;   // gather tile partials [ntiles][4], double-float
   int ntiles = 0;
   float2* Z3C = nullptr;       // thick sources: z-pass coefficient planes [r_z][kxh][Qy]
-  size_t Tq_bytes = 0, YC_bytes = 0, C_bytes = 0, partial_bytes = 0, Z3C_bytes = 0;
+  size_t Tq_bytes = 0, Tqq_bytes = 0, YC_bytes = 0, C_bytes = 0, partial_bytes = 0, Z3C_bytes = 0;
   DftMat yiC;                  // reduced precision: inverse y DFT with the y prefilter
   uint16_t* pkC = nullptr;     // reduced precision: z-mixed coefficient planes, split and packed
   size_t pkC_bytes = 0;
@@ -122,9 +123,10 @@ struct Magnet {
   double Nq_Ms = 0;
   float2* X1 = nullptr;
   float2* YH = nullptr;
-  float* Nq = nullptr;
+  float* Nq = nullptr;   // kernel spectra as planes
+  float* Nqq = nullptr;  // and as quads: which of the two a source has, spectra_forms
   // thick sources (y-forward, z and y-inverse passes): z by a direct sum over
-  // planes (zfft false, nz <= kMaxNzDirect; spectra Nq and Tq as for thin
+  // planes (zfft false, nz <= kMaxNzDirect; spectra Nqq and Tqq as for thin
   // films) or by FFT (grid depth, spectra N3 / S3)
   bool thick = false, zfft = false;
   int Qz = 0, Wz = 0, kzq = 0;
@@ -475,7 +477,7 @@ std::vector<int> plan_pair_radices(int L) {
   long long best_key = -1;
   for (const auto& o : orders) {
     const int m = *std::max_element(o.begin(), o.end());
-    // a first radix below four doubles the twiddle table (fused_pairs counts on 4/3 L)
+    // a first radix below four doubles the twiddle table (pairs_fit counts on 4/3 L)
     if (m > max_r || (o[0] < 4 && *std::max_element(best.begin(), best.end()) >= 4)) continue;
     const long long key = pair_wavefronts(L, o) * 64 + m;
     if (best_key < 0 || key < best_key) {
@@ -765,14 +767,26 @@ int window_needed(const Magnet& S, const Dir& D, int a) {
 // kind 0: the W-folded S spectra of the potential (Tq [n_out][nz][3]);
 // kind 1: the W-folded rows of -N of the componentwise field variant
 // (Tq [3][n_out][nz][3]).
+// The forms of its kernel spectra that a source's passes read (bits): planes for
+// the fused y pass on one column per CTA, quads for that on two and for the plane
+// mixing.  `every`: N, and T of the box of the whole evaluation, which calls of
+// both kinds read (ypass_pairs); else T of a box that coefficient calls alone read.
+constexpr int kPlanes = 1, kQuads = 2;
+int spectra_forms(const Magnet& S, bool every) {
+  if (S.thick) return kQuads;
+  int f = ypass_pairs(S.nz, S.Qy, S.kxh, false) ? kQuads : kPlanes;
+  if (every) f |= ypass_pairs(S.nz, S.Qy, S.kxh, true) ? kQuads : kPlanes;
+  return f;
+}
+
 mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   Magnet& S = ctx->mag[s];
   const int n_out = D->r[2];
   const int bz = D->box_len[2];
   const bool fused = kind == 0 && !S.thick;  // the fused y pass reads it, else the plane mixing pass
-  const bool quads = !fused || fused_pairs(S.nz, S.Qy);
-  const int tstride = quads ? t_stride(S.nz, fused) : 3 * S.nz;
-  if (D->Tq && D->Tq_stride == tstride && D->Tq_quads == quads && D->Tq_box_lo_z == D->box_lo[2] && D->Tq_bz == bz && D->Tq_start_z == D->start[2] &&
+  const int forms = kind == 0 ? spectra_forms(S, D == &S.dir) : kQuads;
+  const int tstride = t_stride(S.nz, fused);
+  if (D->Tq_stride == tstride && D->Tq_forms == forms && D->Tq_box_lo_z == D->box_lo[2] && D->Tq_bz == bz && D->Tq_start_z == D->start[2] &&
       D->Tq_nout == n_out && D->Tq_prefilter == D->prefilter && D->Tq_Q[0] == S.Qx &&
       D->Tq_Q[1] == S.Qy && D->Tq_kind == kind)
     return MM_OK;
@@ -780,9 +794,13 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   CKS(get_fft(ctx, S.Qx, &fx));
   CKS(get_fft(ctx, S.Qy, &fy));
   const size_t qsize = (size_t)S.kxh * S.kyq;
-  const size_t tbytes = sizeof(float) * quad_floats((kind ? 3 : 1) * n_out * tstride, S.kxh, S.kyq);
-  CKS(ensure_buf(ctx, &D->Tq, &D->Tq_bytes, tbytes));
-  CK(cudaMemsetAsync(D->Tq, 0, tbytes, ctx->st));  // the padding of the quads
+  D->Tq_forms = 0;
+  if (forms & kPlanes) CKS(ensure_buf(ctx, &D->Tq, &D->Tq_bytes, sizeof(float) * (size_t)n_out * S.nz * 3 * qsize));
+  if (forms & kQuads) {
+    const size_t tbytes = sizeof(float) * quad_floats((kind ? 3 : 1) * n_out * tstride, S.kxh, S.kyq);
+    CKS(ensure_buf(ctx, &D->Tqq, &D->Tqq_bytes, tbytes));
+    CK(cudaMemsetAsync(D->Tqq, 0, tbytes, ctx->st));  // the padding of the quads
+  }
   // z mixing matrix: rows = output planes, columns = box planes
   std::vector<double> W((size_t)n_out * bz, 0.0);
   double h[kFirHalf + 1];
@@ -804,10 +822,11 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   const KernelPlan K = kernel_plan(ctx, S);
   const double scale = S.Ms / ((double)S.Qx * S.Qy);
   if (kind == 0)
-    CK(build_T_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], scale, D->box_lo[2], bz, n_out, ctx->W_dev, D->Tq,
-                       tstride, quads, ctx->gen_work, ctx->gen_q, ctx->st));
+    CK(build_T_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], scale, D->box_lo[2], bz, n_out, ctx->W_dev,
+                       forms & kPlanes ? D->Tq : nullptr, forms & kQuads ? D->Tqq : nullptr, tstride, ctx->gen_work,
+                       ctx->gen_q, ctx->st));
   else  // H = -N M
-    CK(build_TN_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], -scale, D->box_lo[2], bz, n_out, ctx->W_dev, D->Tq,
+    CK(build_TN_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], -scale, D->box_lo[2], bz, n_out, ctx->W_dev, D->Tqq,
                         ctx->gen_work, ctx->gen_q, ctx->st));
   CK(cudaStreamSynchronize(ctx->st));  // W_dev / scratch reuse
   D->Tq_box_lo_z = D->box_lo[2];
@@ -819,7 +838,7 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   D->Tq_Q[1] = S.Qy;
   D->Tq_kind = kind;
   D->Tq_stride = tstride;
-  D->Tq_quads = quads;
+  D->Tq_forms = forms;
   return MM_OK;
 }
 
@@ -947,10 +966,10 @@ mm_status ensure_plan(mm_ctx* ctx) {
           return fail(ctx, MM_ENOTSUP, "z extent too large for the z pass");
       }
       S.Nq_Ms = 0;  // force a spectra rebuild
-      cudaFree(S.X1); cudaFree(S.YH); cudaFree(S.Nq);
+      cudaFree(S.X1); cudaFree(S.YH); cudaFree(S.Nq); cudaFree(S.Nqq);
       cudaFree(S.N3); cudaFree(S.S3); cudaFree(S.Y3); cudaFree(S.Z3H);
       S.X1 = S.YH = S.Y3 = S.Z3H = nullptr;
-      S.Nq = S.N3 = S.S3 = nullptr;
+      S.Nq = S.Nqq = S.N3 = S.S3 = nullptr;
       S.aux.valid = false;
     }
     const size_t qsize = (size_t)S.kxh * S.kyq;
@@ -958,9 +977,13 @@ mm_status ensure_plan(mm_ctx* ctx) {
       CKS(alloc(ctx, (void**)&S.X1, sizeof(float2) * 3 * S.nz * S.kxh * (size_t)S.ny));
       CKS(alloc(ctx, (void**)&S.YH, sizeof(float2) * 3 * S.nz * S.kxh * (size_t)S.ny));
       if (!S.zfft) {
-        const size_t nbytes = sizeof(float) * quad_floats(6 * S.nz, S.kxh, S.kyq);
-        CKS(alloc(ctx, (void**)&S.Nq, nbytes));
-        CK(cudaMemsetAsync(S.Nq, 0, nbytes, ctx->st));  // the padding of the quads
+        const int forms = spectra_forms(S, true);
+        if (forms & kPlanes) CKS(alloc(ctx, (void**)&S.Nq, sizeof(float) * 6 * S.nz * qsize));
+        if (forms & kQuads) {
+          const size_t nbytes = sizeof(float) * quad_floats(6 * S.nz, S.kxh, S.kyq);
+          CKS(alloc(ctx, (void**)&S.Nqq, nbytes));
+          CK(cudaMemsetAsync(S.Nqq, 0, nbytes, ctx->st));  // the padding of the quads
+        }
       } else {
         CKS(alloc(ctx, (void**)&S.N3, sizeof(float) * 6 * qsize * S.kzq));
         CKS(alloc(ctx, (void**)&S.S3, sizeof(float) * 3 * qsize * S.kzq));
@@ -981,7 +1004,7 @@ mm_status ensure_plan(mm_ctx* ctx) {
                        std::max(ctx->gen_q_bytes, sizeof(double) * 6 * qsize)));
         const KernelPlan K = kernel_plan(ctx, S);
         CK(build_N_spectra(K, fx, fy, S.d[0], S.d[1], S.d[2], -S.Ms / ((double)S.Qx * S.Qy), S.Nq,
-                           S.thick || fused_pairs(S.nz, S.Qy), ctx->gen_work, ctx->gen_q, ctx->st));
+                           S.Nqq, ctx->gen_work, ctx->gen_q, ctx->st));
       } else {
         CKS(build_spectra_3d_all(ctx, S, fx, fy));
       }
@@ -1120,14 +1143,15 @@ mm_status run_source_passes(mm_ctx* ctx, const float* in[2], const int* which, i
       YJob& J = L.job[nj];
       J.in = S.X1;
       J.nz = S.nz; J.ny = S.ny; J.kxh = S.kxh; J.kyq = S.kyq;
-      CKS(get_fft(ctx, S.Qy, &J.fy, fused_pairs(S.nz, S.Qy)));
+      J.pairs = ypass_pairs(S.nz, S.Qy, S.kxh, what[i] == 3) ? 1 : 0;
+      CKS(get_fft(ctx, S.Qy, &J.fy, J.pairs != 0));
       J.do_H = (what[i] & 1) ? 1 : 0;
-      J.Nq = S.Nq;
+      J.Nq = J.pairs ? S.Nqq : S.Nq;
       J.outH = S.YH;
       J.do_C = (what[i] & 2) ? 1 : 0;
       if (J.do_C) {
         J.n_out = D->r[2];
-        J.Tq = D->Tq;
+        J.Tq = J.pairs ? D->Tqq : D->Tq;
         J.outC = D->YC;
         J.box_lo = D->box_lo[1];
         J.box_len = D->box_len[1];
@@ -1210,7 +1234,7 @@ mm_status run_source_passes(mm_ctx* ctx, const float* in[2], const int* which, i
       } else {
         ZMixJob& M = Lm.job[nm];
         M.in = S.Y3; M.nz = S.nz; M.kxh = S.kxh; M.Qy = S.Qy; M.kyq = S.kyq;
-        M.Nq = S.Nq; M.Tq = do_C ? D->Tq : nullptr;
+        M.Nq = S.Nqq; M.Tq = do_C ? D->Tqq : nullptr;
         M.nH = do_H ? P3 : 0;
         M.n_out = do_C ? D->r[2] : 0;
         M.outH = S.Z3H;
@@ -1801,7 +1825,7 @@ static void free_dft(DftMat& M) {
 }
 
 static void free_dir(Dir& D) {
-  cudaFree(D.Tq); cudaFree(D.YC); cudaFree(D.C); cudaFree(D.partial); cudaFree(D.Z3C); cudaFree(D.pkC);
+  cudaFree(D.Tq); cudaFree(D.Tqq); cudaFree(D.YC); cudaFree(D.C); cudaFree(D.partial); cudaFree(D.Z3C); cudaFree(D.pkC);
   free_dft(D.yiC);
   D = Dir();
 }
@@ -1817,7 +1841,7 @@ void mm_destroy(mm_ctx* ctx) {
     for (auto p : M.k) cudaFree(p);
     cudaFree(M.Hself); cudaFree(M.Hstray); cudaFree(M.scratch3); cudaFree(M.err_partial);
     cudaFree(M.pow_H); cudaFree(M.pow_part);
-    cudaFree(M.X1); cudaFree(M.YH); cudaFree(M.Nq);
+    cudaFree(M.X1); cudaFree(M.YH); cudaFree(M.Nq); cudaFree(M.Nqq);
     cudaFree(M.N3); cudaFree(M.S3); cudaFree(M.Y3); cudaFree(M.Z3H);
     free_dft(M.yf); free_dft(M.yiH); cudaFree(M.pkH); cudaFree(M.pkX);
     cudaFree(M.adj_box); cudaFree(M.adj_grid); cudaFree(M.adj_X); cudaFree(M.adj_Y); cudaFree(M.adj_Z);
@@ -2348,7 +2372,7 @@ mm_status mm_compute_stray_field_componentwise(mm_ctx* ctx, int src, float* H_de
     L.njobs = 1;
     ZMixJob& M = L.job[0];
     M.in = S.cw_Y; M.nz = S.nz; M.kxh = S.kxh; M.Qy = S.Qy; M.kyq = S.kyq;
-    M.Nq = S.Nq; M.Tq = D.Tq; M.nH = 0; M.n_out = PC; M.outH = nullptr; M.outC = D.Z3C;
+    M.Nq = nullptr; M.Tq = D.Tqq; M.nH = 0; M.n_out = PC; M.outH = nullptr; M.outC = D.Z3C;
     M.field_nbox = nb;
     L.tile_start[1] = zmix_tiles(S.kxh, S.kyq);
     Timer t(ctx, 8);
@@ -2730,7 +2754,7 @@ mm_status mm_autotune(mm_ctx* ctx, int candidates, int reps, int* n_tuned) {
     classes[S.Qx].insert(0);
     classes[S.Qx].insert(2);
     if (!S.thick) {
-      classes[fused_pairs(S.nz, S.Qy) ? -S.Qy : S.Qy].insert(1);
+      classes[ypass_pairs(S.nz, S.Qy, S.kxh, true) ? -S.Qy : S.Qy].insert(1);
     } else {
       classes[S.Qy].insert(7);
       classes[S.Qy].insert(9);

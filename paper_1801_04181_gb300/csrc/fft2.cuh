@@ -432,6 +432,7 @@ template <int R0, int R1, int R2, int R3 = 1, int PAD = 0> struct CtPair {
 // over its tables cannot differ.  Else the plan at run time.
 template <typename... Plans> struct PairPlans {
   static bool has(const FftPlanDev& P) { return (Plans::is(P) || ...); }
+  static bool has_length(int L) { return ((Plans::kL == L) || ...); }
   // the kernel Pass::build<Fft>() of a launch, whose jobs hold the tables `t`
   template <typename Pass, typename JobT>
   static auto kernel(const Launch<JobT>& L, FftTables JobT::*t) {

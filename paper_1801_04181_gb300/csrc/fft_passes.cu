@@ -260,8 +260,7 @@ __device__ __forceinline__ void ypass_mix(const YJob& J, float2* sm, int kx, int
   }
 }
 
-// One column per CTA: four layers, and lines too long for two columns (fused_pairs);
-// kernel spectra by planes.  Every job of a launch has NZ layers.  kYThreads = 288 (nine
+// One column per CTA (ypass_pairs: where two do not pay); kernel spectra by planes.  Every job of a launch has NZ layers.  kYThreads = 288 (nine
 // warps) covers the 271 frequency pairs of a 540-point line in one round of
 // the spectral products.
 constexpr int kYThreads = 288;
@@ -751,6 +750,35 @@ template <int NZ> struct YPass2 {
 };
 bool ypass_plan_compiled(const FftPlanDev& P) { return YPairPlans::has(P); }
 
+// Whether a source of kxh columns takes two per CTA.  `both`: demag and
+// coefficient planes at once, in a whole evaluation, whose launch takes both
+// films; else planes of one kind of one film.
+//
+// Pairs halve the CTAs and double their shared memory, so they pay where the
+// columns are many against the 152 SMs (one column per CTA: three CTAs a SM up to
+// two layers, two at three) and their lines few and short enough to be taken at
+// once; compiled plans pay further.  The lines are drawn where neither form is
+// slower, from 1200 sizes (20 to 1000 cells in x, 20 to 1024 in y, one to three
+// layers, the three kinds of call).  us of the pass, one column -> two:
+//   short lines: whole evaluations of 300 x 64 x 1 (160 points) 23.5 -> 12.7, 300 x 100 x
+//     3 (240) 34.4 -> 28.5, 145 x 100 x 3 (322 columns) 24.7 -> 23.4, but x 2 16.1 -> 18.1;
+//     40 x 64 x 1 (compiled, few columns) 14.4 -> 10.3, 40 x 100 x 3 (not) 14.4 -> 20.7;
+//   up to 640 points: 600 x 300 x 1 66.6 -> 60.9, 145 x 256 x 1 19.2 -> 20.8; stray field
+//     calls of 450 x 300 x 1 34.8 -> 21.7, x 2 39.1 -> 28.3;
+//   long lines: 600 x 1024 x 1 (2160, compiled) 248 -> 189 whole, 73 -> 82 the stray
+//     field alone; 600 x 400 x 2 (864, planes in five chunks) 130 -> 178.
+constexpr int kSMs = 152;
+bool ypass_pairs(int nz, int Qy, int kxh, bool both) {
+  if (!pairs_fit(nz, Qy)) return false;
+  const bool compiled = YPairPlans::has_length(Qy);
+  const int cols = both ? 2 * kxh : kxh;
+  if (Qy <= 360)
+    return kxh >= 2 * kSMs || (both && nz != 2 && kxh >= kSMs) || (compiled && nz * Qy <= 320);
+  if (nz == 1 && Qy <= 750 && cols >= (Qy > 640 ? 6 : both ? 4 : 3) * kSMs) return true;
+  if (nz == 2 && Qy <= 640 && !both && kxh >= 3 * kSMs && kxh < 6 * kSMs) return true;
+  return compiled && both && (Qy > 640 ? cols >= 6 * kSMs : nz == 2 && cols >= 10 * kSMs);
+}
+
 static size_t ypass2_smem(const YJob& J, int ch) {
   const int n_out = J.do_C ? J.n_out : 0;
   const int cb = J.do_H || ch < n_out ? 3 * J.nz : 0;
@@ -759,7 +787,7 @@ static size_t ypass2_smem(const YJob& J, int ch) {
 }
 
 // Coefficient planes at a time: all of them, or the most that let two CTAs
-// share an SM, or the most that fit (fused_pairs: two at least).  Chunks start on
+// share an SM, or the most that fit (pairs_fit: two at least).  Chunks start on
 // whole quads of the kernel spectra: one layer's hold two planes.
 static int ypass2_chunk(const YJob& J) {
   const int n_out = J.do_C ? J.n_out : 0;
@@ -815,7 +843,7 @@ cudaError_t launch_ypass(const Launch<YJob>& L, size_t smem, cudaStream_t st) {
       Launch<YJob> S{};
       int tiles = 0;
       for (int i = 0; i < L.njobs; ++i) {
-        if (L.job[i].nz != nz || fused_pairs(nz, L.job[i].fy.plan.L) != (pairs != 0)) continue;
+        if (L.job[i].nz != nz || L.job[i].pairs != pairs) continue;
         S.job[S.njobs] = L.job[i];
         S.tile_start[S.njobs] = tiles;
         tiles += L.job[i].kxh;

@@ -283,9 +283,10 @@ __global__ void k_extract_quarter(const double2* spec, double* out, int Qx, int 
 }
 
 // T[o][jz][c] = scale * sum_zb W[o][zb] Sq[(zb - jz) - dz_lo][c]  (quarter
-// planes), plane o * tstride + jz * 3 + c, as quads or by planes
-__global__ void k_mix_T(const double* Sq, const double* W, float* T, int n_out, int nz, int bz,
-                        int dz_first_plane_offset, int kxh, int kyq, int tstride, int quads, double scale) {
+// planes): into plane oj * 3 + c of `planes` and plane o * qstride + jz * 3 + c of
+// `quads` (either may be null)
+__global__ void k_mix_T(const double* Sq, const double* W, float* planes, float* quads, int n_out, int nz, int bz,
+                        int dz_first_plane_offset, int kxh, int kyq, int qstride, double scale) {
   const size_t qsize = (size_t)kxh * kyq;
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= qsize) return;
@@ -299,8 +300,9 @@ __global__ void k_mix_T(const double* Sq, const double* W, float* T, int n_out, 
     const int plane = zb - jz + dz_first_plane_offset;
     acc += w * Sq[((size_t)plane * 3 + c) * qsize + i];
   }
-  const int p = o * tstride + jz * 3 + c;
-  T[quads ? quad_index(p, (int)(i / kyq), (int)(i % kyq), kxh, kyq) : (size_t)p * qsize + i] = (float)(scale * acc);
+  const float t = (float)(scale * acc);
+  if (planes) planes[(size_t)(oj * 3 + c) * qsize + i] = t;
+  if (quads) quads[quad_index(o * qstride + jz * 3 + c, (int)(i / kyq), (int)(i % kyq), kxh, kyq)] = t;
 }
 
 // Componentwise field variant: TN[(a n_out + o) nz + jz][b] = scale * sum_zb
@@ -327,11 +329,13 @@ __global__ void k_mix_TN(const double* Nq6, const double* W, float* T, int n_out
       (float)(scale * acc);
 }
 
-// one quarter plane into plane `plane` of an array of quads or planes
-__global__ void k_put_plane(const double* in, float* out, int plane, int kxh, int kyq, int quads, double scale) {
+// one quarter plane into plane `plane` of an array of planes and one of quads (either may be null)
+__global__ void k_put_plane(const double* in, float* planes, float* quads, int plane, int kxh, int kyq, double scale) {
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x, n = (size_t)kxh * kyq;
-  if (i < n)
-    out[quads ? quad_index(plane, (int)(i / kyq), (int)(i % kyq), kxh, kyq) : plane * n + i] = (float)(scale * in[i]);
+  if (i >= n) return;
+  const float v = (float)(scale * in[i]);
+  if (planes) planes[plane * n + i] = v;
+  if (quads) quads[quad_index(plane, (int)(i / kyq), (int)(i % kyq), kxh, kyq)] = v;
 }
 
 __global__ void k_scale_to_float(const double* in, float* out, size_t n, double scale) {
@@ -382,7 +386,7 @@ static cudaError_t plane_spectra(int kind, int ncomp, const KernelPlan& K, int d
 }
 
 cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
-                            double b, double c, double scale, float* Nq, bool quads, double2* work, double* qbuf,
+                            double b, double c, double scale, float* planes, float* quads, double2* work, double* qbuf,
                             cudaStream_t st) {
   const int kxh = K.Qx / 2 + 1, kyq = K.Qy / 2 + 1;
   const size_t qsize = (size_t)kxh * kyq;
@@ -391,8 +395,8 @@ cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftT
     cudaError_t e = plane_spectra(1, 6, K, dz, a, b, c, fx, fy, work, qbuf, imag6, st);
     if (e != cudaSuccess) return e;
     for (int q = 0; q < 6; ++q)
-      k_put_plane<<<(unsigned)((qsize + 255) / 256), 256, 0, st>>>(qbuf + q * qsize, Nq, dz * 6 + q, kxh, kyq, quads,
-                                                                        scale);
+      k_put_plane<<<(unsigned)((qsize + 255) / 256), 256, 0, st>>>(qbuf + q * qsize, planes, quads, dz * 6 + q, kxh,
+                                                                   kyq, scale);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -401,7 +405,7 @@ cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftT
 
 cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                             double b, double c, double scale, int box_lo_z, int bz, int n_out,
-                            const double* W_dev, float* Tq, int tstride, bool quads, double2* work, double* Sq,
+                            const double* W_dev, float* planes, float* quads, int qstride, double2* work, double* Sq,
                             cudaStream_t st) {
   const int kxh = K.Qx / 2 + 1, kyq = K.Qy / 2 + 1;
   const size_t qsize = (size_t)kxh * kyq;
@@ -415,7 +419,7 @@ cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftT
   }
   // plane index of offset dz = (box_lo_z + zb) - jz is (zb - jz) + (nz - 1)
   dim3 g((unsigned)((qsize + 255) / 256), 3, n_out * K.nz);
-  k_mix_T<<<g, 256, 0, st>>>(Sq, W_dev, Tq, n_out, K.nz, bz, K.nz - 1, kxh, kyq, tstride, quads, scale);
+  k_mix_T<<<g, 256, 0, st>>>(Sq, W_dev, planes, quads, n_out, K.nz, bz, K.nz - 1, kxh, kyq, qstride, scale);
   return cudaGetLastError();
 }
 

@@ -48,14 +48,14 @@ __host__ __device__ inline size_t quad_index(int plane, int kx, int ky, int kxh,
 __host__ __device__ inline size_t quad_floats(int planes, int kxh, int kyq) {
   return (size_t)((planes + 1) >> 1) * ((kxh + 1) >> 1) * kyq * 4;
 }
-// Whether the fused y pass takes two columns per CTA: up to three layers (four
-// spill its 80 registers: 400 x 200 x 4 181 -> 229 us a call) where the lines of the
-// inputs and two outputs fit a CTA's shared memory beside the tables (twiddles
-// at most 4/3 Qy: pair plans start with a radix of four or more; prefilter
-// indices at most Qy + 37).  Its kernel spectra are quads
-// then; for one column per CTA they are planes [plane][kx][ky], plane numbers alike
-// with 3 nz planes per output of T.
-__host__ __device__ constexpr bool fused_pairs(int nz, int Qy) {
+// Whether the fused y pass can take two columns per CTA (ypass_pairs: whether it
+// does): up to three layers (four spill its 80 registers: 400 x 200 x 4 181 -> 229 us
+// a call) where the lines of the inputs and two outputs fit a CTA's shared memory
+// beside the tables (twiddles at most 4/3 Qy: pair plans start with a radix of four
+// or more; prefilter indices at most Qy + 37).  Its kernel spectra are quads; the
+// pass on one column per CTA reads planes [plane][kx][ky], plane numbers alike with
+// 3 nz planes per output of T.
+__host__ __device__ constexpr bool pairs_fit(int nz, int Qy) {
   return nz <= 3 && (size_t)(3 * nz + 2) * Qy * 16 + 26 * (size_t)Qy + 512 <= 227 * 1024;
 }
 // planes of N: dz * 6 + component; planes of T: o * stride + jz * 3 + c, the
@@ -97,7 +97,8 @@ struct YJob {
   int kyq;                // Qy/2 + 1 stored ky values of the kernel spectra
   // self-demag output
   int do_H;
-  const float* Nq;        // quads or planes (fused_pairs), dz * 6 + (xx yy zz xy xz yz), dz >= 0
+  int pairs;              // two columns per CTA; Nq, Tq and fy are of that form
+  const float* Nq;        // quads (pairs) or planes, dz * 6 + (xx yy zz xy xz yz), dz >= 0
   float2* outH;           // [3 nz][kxh][ny]
   // potential / coefficient output
   int do_C;
@@ -405,6 +406,7 @@ cudaError_t init_fft_constants_kgen();
 cudaError_t init_fft_constants_3d();
 size_t ypass_table_bytes(int r);
 bool ypass_plan_compiled(const FftPlanDev& P);  // the y pass on column pairs has a build of this plan
+bool ypass_pairs(int nz, int Qy, int kxh, bool both);
 cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st);
 cudaError_t launch_ypass(const Launch<YJob>& L, size_t smem, cudaStream_t st);
 cudaError_t launch_xinv(const Launch<XInvJob>& L, int Qmax, cudaStream_t st);
@@ -474,7 +476,7 @@ cudaError_t launch_mech(const MechParams& P, cudaStream_t st);
 cudaError_t eval_points_fp64(int kind, int n, const double* off_dev, double a, double b, double c,
                              double* out_dev, cudaStream_t st);
 cudaError_t build_N_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
-                            double b, double c, double scale, float* Nq, bool quads, double2* work, double* qbuf,
+                            double b, double c, double scale, float* planes, float* quads, double2* work, double* qbuf,
                             cudaStream_t st);
 // 3D spectra of S (kind 0, 3 comps) or N (kind 1, 6 comps): out [comp][kxh][kyq][kzq].
 // Scratch: work 2 * ncomp * Qx * Qy double2, q2 ncomp * Qz * kxh * kyq double,
@@ -496,7 +498,7 @@ cudaError_t build_S_planes(const KernelPlan& K, const FftTables& fx, const FftTa
                            double* qtmp, cudaStream_t st);
 cudaError_t build_T_spectra(const KernelPlan& K, const FftTables& fx, const FftTables& fy, double a,
                             double b, double c, double scale, int box_lo_z, int bz, int n_out,
-                            const double* W_dev, float* Tq, int tstride, bool quads, double2* work, double* Sq,
+                            const double* W_dev, float* planes, float* quads, int qstride, double2* work, double* Sq,
                             cudaStream_t st);
 
 }  // namespace mm
