@@ -287,10 +287,10 @@ __device__ __forceinline__ void fft2_stage(const G& g, float4* buf, int ldl, int
 // The first stage of a decimation-in-frequency transform, the points n0 + k M
 // of a butterfly of line l read through ld(l, n0, M, v); twiddles from the
 // plan's global table (coalesced).
-template <int R, int MODE, typename G, typename Ld>
+template <int R, typename G, typename Ld>
 __device__ __forceinline__ void fft2_first(const G& g, float4* buf, int ldl, int nlines,
                                            const float2* __restrict__ tw, Ld ld) {
-  constexpr int S = MODE == kFwdDif ? -1 : 1;
+  constexpr int S = -1;
   const int M = g.M();
   fft2_butterflies(g, nlines, [&](int line, int n0, int n1) {
     c2 v[R];
@@ -331,18 +331,18 @@ __device__ __forceinline__ void fft2_last(const G& g, const float4* buf, int ldl
 // compiled in) ...
 template <unsigned RSET> struct RtPair {
   static constexpr int kL = 0;
-  // Decimation-in-frequency transforms (kFwdDif, kInvDif) of `nlines` lines of
+  // Forward (decimation-in-frequency) transforms of `nlines` lines of
   // buf (stride ldl): line l's points come from ld(l, n0, M, v); then also()
   // runs, before the first barrier (it may fill tw, the pair table, and what
   // else is needed later, while the first loads are on their way).  Ends with a
   // barrier.
-  template <int MODE, typename Ld, typename Also>
+  template <typename Ld, typename Also>
   static __device__ __forceinline__ void in(float4* buf, int ldl, int nlines, const FftTables& T, const float4* tw,
                                             Ld ld, Also also) {
     const FftPlanDev& P = T.plan;
     switch (P.radix[0]) {
 #define MM_STAGE(R) \
-  case R: if constexpr ((RSET & radix_bit(R)) != 0u) fft2_first<R, MODE>(RtStage<R>(P, 0), buf, ldl, nlines, T.tw_f, ld); break;
+  case R: if constexpr ((RSET & radix_bit(R)) != 0u) fft2_first<R>(RtStage<R>(P, 0), buf, ldl, nlines, T.tw_f, ld); break;
       MM_RADICES(MM_STAGE)
 #undef MM_STAGE
       default: break;
@@ -353,7 +353,7 @@ template <unsigned RSET> struct RtPair {
       const float4* ts = tw + T.tw2_off[s];
       switch (P.radix[s]) {
 #define MM_STAGE(R) \
-  case R: if constexpr ((RSET & radix_bit(R)) != 0u) fft2_stage<R, MODE>(RtStage<R>(P, s), buf, ldl, nlines, ts); break;
+  case R: if constexpr ((RSET & radix_bit(R)) != 0u) fft2_stage<R, kFwdDif>(RtStage<R>(P, s), buf, ldl, nlines, ts); break;
         MM_RADICES(MM_STAGE)
 #undef MM_STAGE
         default: break;
@@ -397,18 +397,18 @@ template <int R0, int R1, int R2, int R3 = 1, int PAD = 0> struct CtPair {
     return P.nstages == (R3 > 1 ? 4 : 3) && P.radix[0] == R0 && P.radix[1] == R1 && P.radix[2] == R2 &&
            (R3 == 1 || P.radix[3] == R3);
   }
-  template <int MODE, typename Ld, typename Also>
+  template <typename Ld, typename Also>
   static __device__ __forceinline__ void in(float4* buf, int, int nlines, const FftTables& T, const float4* tw, Ld ld,
                                             Also also) {
-    fft2_first<R0, MODE>(CtStage<R0, kL, kL>(), buf, ldl, nlines, T.tw_f, ld);
+    fft2_first<R0>(CtStage<R0, kL, kL>(), buf, ldl, nlines, T.tw_f, ld);
     also();
     __syncthreads();
-    fft2_stage<R1, MODE>(CtStage<R1, kL, R1 * R2 * R3>(), buf, ldl, nlines, tw + T.tw2_off[1]);
+    fft2_stage<R1, kFwdDif>(CtStage<R1, kL, R1 * R2 * R3>(), buf, ldl, nlines, tw + T.tw2_off[1]);
     __syncthreads();
-    fft2_stage<R2, MODE>(CtStage<R2, kL, R2 * R3>(), buf, ldl, nlines, tw + T.tw2_off[2]);
+    fft2_stage<R2, kFwdDif>(CtStage<R2, kL, R2 * R3>(), buf, ldl, nlines, tw + T.tw2_off[2]);
     __syncthreads();
     if constexpr (R3 > 1) {
-      fft2_stage<R3, MODE>(CtStage<R3, kL, R3>(), buf, ldl, nlines, tw);
+      fft2_stage<R3, kFwdDif>(CtStage<R3, kL, R3>(), buf, ldl, nlines, tw);
       __syncthreads();
     }
   }
@@ -433,7 +433,8 @@ template <int R0, int R1, int R2, int R3 = 1, int PAD = 0> struct CtPair {
 template <typename... Plans> struct PairPlans {
   static bool has(const FftPlanDev& P) { return (Plans::is(P) || ...); }
   static bool has_length(int L) { return ((Plans::kL == L) || ...); }
-  // the kernel Pass::build<Fft>() of a launch, whose jobs hold the tables `t`
+  // the kernel Pass::build<Fft>() of a launch, whose jobs hold the tables `t`;
+  // lengths that never reach the pass (Pass::takes) get no build
   template <typename Pass, typename JobT>
   static auto kernel(const Launch<JobT>& L, FftTables JobT::*t) {
     unsigned rs = 0;
@@ -445,7 +446,11 @@ template <typename... Plans> struct PairPlans {
         if (!is((L.job[i].*t).plan)) return false;
       return true;
     };
-    ((void)(all(&Plans::is) ? (void)(k = Pass::template build<Plans>()) : (void)0), ...);
+    auto take = [&](auto plan) {
+      if constexpr (Pass::takes(decltype(plan)::kL))
+        if (all(&decltype(plan)::is)) k = Pass::template build<decltype(plan)>();
+    };
+    (take(Plans()), ...);
     return k;
   }
 };

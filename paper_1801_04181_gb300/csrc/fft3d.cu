@@ -140,7 +140,7 @@ __global__ void __launch_bounds__(kZThreads, 2) k_zpass3(const Launch<ZJob> Lc) 
   // the 3 nz values of a y position are one run in memory, nz of each
   // component; layers [nz, Qz) are zero padding
   const float2* src = J.in + ((size_t)kx * Qy + y0) * P3;
-  Fft::template in<kFwdDif>(
+  Fft::in(
       sm4, ldz, nin, J.fz, tws,
       [&](int l, int z0, int M, auto& v) {
         const int tp = l / 3, c = l - 3 * tp;
@@ -535,9 +535,11 @@ cudaError_t launch_yfwd3(const Launch<YFwdJob>& L, cudaStream_t st) {
   return launch_chained(k, grid, 256, smem, st, L);
 }
 
-// the lengths of 64 and 128 layers, their plans as constants
+// the lengths of 64 and 128 layers, their plans as constants: 64 x 64 x 64 228 -> 209
+// us, 64 x 64 x 128 427 -> 391 us a launch
 using ZPairPlans = PairPlans<CtPair<4, 8, 5, 1, 1>, CtPair<4, 8, 9, 1, 1>>;
 struct ZPass3 {
+  static constexpr bool takes(int) { return true; }
   template <typename Fft> static auto build() { return &k_zpass3<Fft>; }
 };
 

@@ -493,7 +493,7 @@ __global__ void __launch_bounds__(kY2Threads, 1) k_ypass2(const Launch<YJob> Lc)
     // rows [ny, Q) are zero padding; column b follows column a
     const float2* ca = J.in + (size_t)kxa * ny;
     const int nb = has_b ? ny : 0;
-    Fft::template in<kFwdDif>(
+    Fft::in(
         sm4, Q, Pin, J.fy, tws,
         [&](int p, int y0, int M, auto& v) {
           const float2* src = ca + p * pstride + y0;
@@ -741,11 +741,16 @@ cudaError_t launch_xfwd(const Launch<XFwdJob>& L, int Qmax, cudaStream_t st) {
 // fit shared memory.
 constexpr size_t kSmemTwo = (228 * 1024) / 2 - 1024;  // each of two CTAs on an SM
 
-// the lengths of 64, 128, 256, 512 and 1024 cells (4 cells of margin) with
-// their plans as constants, 13% faster at 540
+// the lengths of 64, 128, 256, 512 and 1024 cells (4 cells of margin) with their
+// plans as constants.  us of whole evaluations' launches, plan at run time ->
+// constant: 300 x 64 x 1 (160 points) 14.0 -> 12.5, 300 x 128 x 2 (288) 25.6 -> 24.8,
+// 1024 x 256 x 2 (540) 110 -> 94, 450 x 512 x 1 (1080) 79 -> 64 and x 3 213 -> 198,
+// 1024 x 1024 x 1 (2160) 328 -> 300
 using YPairPlans =
     PairPlans<CtPair<4, 8, 5>, CtPair<4, 8, 9>, CtPair<12, 9, 5>, CtPair<10, 12, 9>, CtPair<6, 8, 9, 5>>;
 template <int NZ> struct YPass2 {
+  // three layers: short lines, and 1080 points (ypass_pairs)
+  static constexpr bool takes(int L) { return pairs_fit(NZ, L) && (NZ < 3 || L <= 360 || L > 640); }
   template <typename Fft> static auto build() { return &k_ypass2<NZ, Fft>; }
 };
 bool ypass_plan_compiled(const FftPlanDev& P) { return YPairPlans::has(P); }
