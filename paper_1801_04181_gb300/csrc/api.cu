@@ -82,6 +82,7 @@ struct Dir {
   int start[3] = {0, 0, 0}, r[3] = {0, 0, 0}, guard[3] = {0, 0, 0};
   int Tq_box_lo_z = 0, Tq_bz = 0, Tq_start_z = 0, Tq_nout = 0, Tq_prefilter = -1, Tq_Q[2] = {0, 0};
   int Tq_kind = 0;             // 0: S (potential); 1: rows of -N (componentwise field variant)
+  double Tq_Ms = 0;            // the spectra carry the source's Ms
   int Tq_stride = 0;           // planes per output of the quads
   int Tq_forms = 0;            // the forms held: bit 1 planes, bit 2 quads
   float* Tq = nullptr;         // planes
@@ -788,7 +789,7 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   const int tstride = t_stride(S.nz, fused);
   if (D->Tq_stride == tstride && D->Tq_forms == forms && D->Tq_box_lo_z == D->box_lo[2] && D->Tq_bz == bz && D->Tq_start_z == D->start[2] &&
       D->Tq_nout == n_out && D->Tq_prefilter == D->prefilter && D->Tq_Q[0] == S.Qx &&
-      D->Tq_Q[1] == S.Qy && D->Tq_kind == kind)
+      D->Tq_Q[1] == S.Qy && D->Tq_kind == kind && D->Tq_Ms == S.Ms)
     return MM_OK;
   FftTables fx, fy;
   CKS(get_fft(ctx, S.Qx, &fx));
@@ -837,6 +838,7 @@ mm_status build_T(mm_ctx* ctx, int s, Dir* D, int kind = 0) {
   D->Tq_Q[0] = S.Qx;
   D->Tq_Q[1] = S.Qy;
   D->Tq_kind = kind;
+  D->Tq_Ms = S.Ms;
   D->Tq_stride = tstride;
   D->Tq_forms = forms;
   return MM_OK;
@@ -1912,10 +1914,6 @@ mm_status mm_set_material(mm_ctx* ctx, int mag, double Ms, double Aex, double Ku
   M.mat = true;
   ctx->planned = false;
   ctx->k1_valid = false;
-  // spectra carry Ms: force a rebuild of this source's kernels
-  M.Nq_Ms = 0;
-  M.dir.Tq_prefilter = -1;
-  M.aux.Tq_prefilter = -1;
   return MM_OK;
 }
 
