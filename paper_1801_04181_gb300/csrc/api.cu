@@ -1015,6 +1015,11 @@ mm_status ensure_plan(mm_ctx* ctx) {
     }
     if (!S.zfft) CKS(build_T(ctx, s, &D));
     CKS(alloc_dir_outputs(ctx, s, &D));
+    // the tables of the passes on pair lines too: a call may be the first of its
+    // kind under stream capture, where nothing can be allocated
+    FftTables pairs;
+    if (!S.thick && (spectra_forms(S, true) & kQuads)) CKS(get_fft(ctx, S.Qy, &pairs, true));
+    if (S.zfft) CKS(get_fft(ctx, S.Qz, &pairs, true));
     D.valid = true;
   }
   ctx->planned = true;
