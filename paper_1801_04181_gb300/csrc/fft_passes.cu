@@ -466,10 +466,9 @@ __device__ __forceinline__ void ypass2_mix(const YJob& J, float4* sm, int kxp, i
 // What bounds it: shared memory and the latency of the kernel spectra between
 // the barriers (stick-slip films: 46% of the shared-memory wavefronts, 40%
 // issue-active, 20% DRAM).  Against the one-column pass, 40 M warp instructions
-// for 64 M and 94 -> 92 us there; one 1024 x 1024 film over another (one CTA
-// per SM in both) 411 -> 322 us, 355 x 145 x 3 over 301 x 127 x 2 37 + 26 -> 26 +
-// 23 us, 64 x 64 x 1 19 -> 13 us.  640 or 512 threads per SM (fewer, with more
-// registers) measured 0-10% slower over these sizes.
+// for 64 M and 94 -> 92 us there; other sizes beside the rule (ypass_pairs).  640
+// or 512 threads per SM (fewer, with more registers) measured 0-10% slower over
+// 64 x 64 x 1, 355 x 145 x 3, 1024 x 256 x 2 and 1024 x 1024 x 1.
 constexpr int kY2Threads = 768;  // per SM, shared out over its CTAs
 template <int NZ, typename Fft>
 __global__ void __launch_bounds__(kY2Threads, 1) k_ypass2(const Launch<YJob> Lc) {
